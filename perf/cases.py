@@ -65,7 +65,7 @@ def listed():
         # an odd-sized photograph, 16-bit storage of the corrections
         {"name": "poisson_odd", "kind": "poisson", "w": 1355, "h": 757, "c": 3,
          "storage": "bf16", "mask": False, "nu1": 2, "nu2": 1},
-        # thresholded Laplacian field at 4K, one channel
+        # a splatted Laplacian field at 4K with the hard threshold, one channel
         {"name": "rho_4k", "kind": "rho", "w": 3840, "h": 2160, "c": 1, "storage": "f16",
          "threshold": 0.004},
         # one view of the training workload: forward, loss, backward
@@ -170,7 +170,19 @@ def _poisson_inputs(case, seed):
 
 
 def _rho_input(case, seed):
-    return _divergence(_gradient_maps(_photo(case["c"], case["h"], case["w"], seed))).contiguous()
+    """A Laplacian field as splats give it: sparse blobs a few pixels wide with Laplace
+    amplitudes, whose sum is not zero."""
+    c, h, w = case["c"], case["h"], case["w"]
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    u = torch.rand((c, h, w), generator=gen, device="cuda") * 2.0 - 1.0
+    amp = -0.05 * torch.sign(u) * torch.log1p(-u.abs().clamp_max(1.0 - 1e-6))
+    rho = amp * (torch.rand((c, h, w), generator=gen, device="cuda") < 0.01)
+    tap = torch.exp(-(torch.arange(-8, 9, device="cuda") ** 2) / 18.0).tolist()
+    for dim, size in ((1, h), (2, w)):
+        pad = torch.nn.functional.pad(rho, (8, 8, 0, 0) if dim == 2 else (0, 0, 8, 8))
+        rho = sum(t * pad.narrow(dim, k, size) for k, t in enumerate(tap))
+    return rho.contiguous()
 
 
 def _requests(case, seed):
