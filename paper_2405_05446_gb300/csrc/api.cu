@@ -434,6 +434,7 @@ static int poisson_common(const float *field, int input_is_rho, const uint8_t *t
   a.nu2 = so.nu2;
   a.omega = so.omega;
   a.storage = so.storage;
+  a.coarse_max_dim = so.coarse_max_dim;
   a.max_cycles = so.max_cycles;
   a.rtol = so.rtol;
   a.plan = &p;
@@ -494,6 +495,7 @@ static int render_view_impl(const gdgs_gaussians *g, const gdgs_camera *cam,
   a.nu2 = so.nu2;
   a.omega = so.omega;
   a.storage = so.storage;
+  a.coarse_max_dim = so.coarse_max_dim;
   a.max_cycles = so.max_cycles;
   a.rtol = so.rtol;
   a.plan = &p;
@@ -559,6 +561,7 @@ int gdgs_render_view_backward(const gdgs_gaussians *g, const gdgs_camera *cam,
   a.nu2 = so.nu2;
   a.omega = so.omega;
   a.storage = so.storage;
+  a.coarse_max_dim = so.coarse_max_dim;
   a.max_cycles = so.max_cycles;
   a.rtol = so.rtol;
   a.plan = &pa;
@@ -630,6 +633,24 @@ int gdgs_sync_status(const void *ws, gdgs_solve_stats *stats, void *stream) {
   if (cudaMemcpy(&c, ws, sizeof(Ctrl), cudaMemcpyDeviceToHost) != cudaSuccess) return GDGS_ERR_CUDA;
   int status = c.status;
   double rel = 0.0;
+  if (c.direct > 0) {  // a direct solve: per-channel residuals
+    const double thr = c.rtol * c.rtol;
+    double r0 = 0.0, rf = 0.0;
+    bool met = true;
+    c.cycles = 0;
+    for (int i = 0; i < c.channels && i < GDGS_MAX_CHANNELS; ++i) {
+      const int kf = c.kf_c[i];
+      if (kf < 0 || kf > c.direct) return GDGS_ERR_CUDA;  // not a finished solve's block
+      const double a = c.rnorm2[fct_slot(0, i)], b = c.rnorm2[fct_slot(kf, i)];
+      r0 += a;
+      rf += b;
+      met = met && b <= thr * a;
+      if (kf > c.cycles) c.cycles = kf;
+    }
+    c.rnorm2[0] = r0;
+    c.final_rnorm2 = rf;
+    c.stopped = met;
+  }
   if (c.max_cycles > 0) {  // a solve ran
     const double r0 = c.rnorm2[0];
     rel = r0 > 0 ? sqrt(c.final_rnorm2 / r0) : 0.0;

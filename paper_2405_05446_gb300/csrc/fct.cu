@@ -1,0 +1,300 @@
+// Direct Neumann solve (Eq. p2d) by cosine transforms, refined to the caller's rtol.
+// Measured on a GB300 against the multigrid cycles it takes over from: 1920x1080x3 from
+// maps 743 -> 221 us, 1355x757x3 (Bluestein) 779 -> 350 us, 3840x2160x1 1486 -> 301 us,
+// 128x96x1 220 -> 59 us; relative error of the image 1.7e-6 -> 7e-8 (1080p).
+//
+// On the pixel grid the 5-point Neumann Laplacian is diagonal in the DCT-II modes of
+// the two sides (Sec. 2.1 lists Fourier-type solvers beside multigrid): with
+// lambda(ky, kx) = -4 sin^2(pi ky / 2H) - 4 sin^2(pi kx / 2W), e = IDCT(DCT(r) / lambda)
+// solves L e = r exactly up to FP32 rounding. One cycle is three passes over the image:
+//   rows      residual r of the current iterate, its DCT along x        -> spectrum
+//   columns   DCT along y, the division by lambda, inverse DCT along y  -> spectrum
+//   rows back inverse DCT along x, u += e (float-float)
+// FP32 rounding of e leaves a relative residual of ~1e-5 (it is the size of the image's
+// own FP32 representation error), and the next cycle solves for exactly that: the
+// residual is evaluated from the float-float iterate with error-free sums, so two cycles
+// reach ~1e-7 or less. The multigrid needs 4-6 cycles, each a chain of ~12 dependent
+// launches whose small levels leave the GPU idle (1080p, three channels: 150 us per
+// cycle, all latency); here every launch covers all channels and every SM.
+//
+// A transform of n points works on two real sequences at once, packed as the real and
+// imaginary part of one complex FFT of n points (Makhoul's even-odd order), held in
+// shared memory. The FFT is mixed-radix Stockham, one radix-R butterfly set per thread
+// in registers between two barriers, in place. Sides with a prime factor above 13 use
+// Bluestein's chirp convolution on a length >= 2 n - 1 instead.
+#include <stdlib.h>
+
+#include <algorithm>
+#include <atomic>
+#include <vector>
+
+#include "fct.cuh"
+
+namespace gdgs {
+
+const FctKernels *fct_slice0(int *);
+const FctKernels *fct_slice1(int *);
+const FctKernels *fct_slice2(int *);
+const FctKernels *fct_slice3(int *);
+const FctKernels *fct_slice4(int *);
+const FctKernels *fct_slice5(int *);
+const FctKernels *fct_slice6(int *);
+const FctKernels *fct_slice7(int *);
+const FctKernels *fct_slice8(int *);
+const FctKernels *fct_slice9(int *);
+const FctKernels *fct_slice10(int *);
+const FctKernels *fct_slice11(int *);
+const FctKernels *fct_slice12(int *);
+const FctKernels *fct_slice13(int *);
+const FctKernels *fct_slice14(int *);
+const FctKernels *fct_slice15(int *);
+
+namespace {
+
+// After `k` cycles: image = u + (m_c - mean u) of the iterate channel c stopped at, and
+// (when that is the k-th) its residual. Skipped when an earlier call already finished c.
+template <int V>
+__global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant__ FctArgs a, int k, int first) {
+  griddep_enter();
+  const int c = blockIdx.y;
+  __shared__ int s_kf, s_skip;
+  __shared__ float s_shift;
+  if (threadIdx.x == 0) {
+    bool done;
+    const int kf = fct_cycles_done(a.ctrl, c, a.inv_cells, k - 1, &done);
+    s_skip = done && !first;
+    s_kf = done ? kf : k;
+    float mc = a.mean[0];
+#pragma unroll
+    for (int i = 1; i < GDGS_MAX_CHANNELS; ++i)
+      if (i == c) mc = a.mean[i];
+    s_shift = (float)((double)mc - a.ctrl->sum_u[s_kf][c] * a.inv_cells);
+    if (blockIdx.x == 0 && !s_skip) {
+      a.ctrl->kf_c[c] = s_kf;
+      a.ctrl->mean_set[c] = mc;
+      a.ctrl->rnorm2[fct_slot(0, c)] = fct_r0(a.ctrl, c, a.inv_cells);
+    }
+  }
+  __syncthreads();
+  if (s_skip) return;
+  const FctMean mr = fct_block_mean(a, c);
+  const int kf = s_kf, W = a.W, H = a.H;
+  const float shift = s_shift;
+  const size_t plane = (size_t)H * W;
+  const float *rho = a.rho + c * plane, *uh = a.uhi + c * plane, *ul = a.ulo + c * plane;
+  float *img = a.image + c * plane;
+  float r2 = 0.f;
+  const int Wq = W / V;
+  const long long nq = (long long)H * Wq;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nq; q += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(q / Wq), j0 = (int)(q - (long long)i * Wq) * V;
+    const size_t p = (size_t)i * W + j0;
+    if (kf == 0) {
+#pragma unroll
+      for (int d = 0; d < V; ++d) img[p + d] = 0.f + (0.f + shift);
+      continue;
+    }
+    const size_t ps = i + 1 < H ? p + W : p, pn = i > 0 ? p - W : p;
+    float h[V + 2], l[V + 2], hs[V], ls[V], hn[V], ln[V], rv[V];
+    const bool low = kf > 1;
+    auto row = [&](const float *src, size_t o, float *dst) {
+      if constexpr (V == 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(src + o));
+        dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w;
+      } else {
+        dst[0] = __ldg(src + o);
+      }
+    };
+    row(rho, p, rv);
+    row(uh, p, h + 1);
+    row(uh, ps, hs);
+    row(uh, pn, hn);
+    h[0] = j0 > 0 ? __ldg(uh + p - 1) : h[1];
+    h[V + 1] = j0 + V < W ? __ldg(uh + p + V) : h[V];
+#pragma unroll
+    for (int d = 0; d < V; ++d) l[d + 1] = ls[d] = ln[d] = 0.f;
+    l[0] = l[V + 1] = 0.f;
+    if (low) {
+      row(ul, p, l + 1);
+      row(ul, ps, ls);
+      row(ul, pn, ln);
+      l[0] = j0 > 0 ? __ldg(ul + p - 1) : l[1];
+      l[V + 1] = j0 + V < W ? __ldg(ul + p + V) : l[V];
+    }
+    float o[V];
+    FctDiff west = fct_diff<true>(h[1], l[1], h[0], l[0]);
+#pragma unroll
+    for (int d = 0; d < V; ++d) {
+      const FctDiff east = fct_diff<true>(h[d + 2], l[d + 2], h[d + 1], l[d + 1]);
+      const FctDiff south = fct_diff<true>(hs[d], ls[d], h[d + 1], l[d + 1]);
+      const FctDiff north = fct_diff<true>(h[d + 1], l[d + 1], hn[d], ln[d]);
+      const float r = fct_residual(rv[d], mr.hi, mr.lo, east, west, south, north);
+      r2 = fmaf(r, r, r2);
+      o[d] = h[d + 1] + (l[d + 1] + shift);
+      west = east;
+    }
+    if constexpr (V == 4) *reinterpret_cast<float4 *>(img + p) = make_float4(o[0], o[1], o[2], o[3]);
+    else img[p] = o[0];
+  }
+  r2 = fct_block_sum(r2);
+  if (threadIdx.x == 0 && kf == k) atomicAdd(&a.ctrl->rnorm2[fct_slot(k, c)], (double)r2);
+}
+
+// ------------------------------------------------------------------ plans (host)
+
+// Every FFT length, ascending, the direct ones before the Bluestein ones.
+const std::vector<FctKernels> &lengths() {
+  static const std::vector<FctKernels> all = [] {
+    const FctKernels *(*slices[kFctSlices])(int *) = {fct_slice0, fct_slice1, fct_slice2, fct_slice3, fct_slice4, fct_slice5, fct_slice6, fct_slice7, fct_slice8, fct_slice9, fct_slice10, fct_slice11, fct_slice12, fct_slice13, fct_slice14, fct_slice15};
+    std::vector<FctKernels> v;
+    for (auto s : slices) {
+      int n = 0;
+      const FctKernels *e = s(&n);
+      v.insert(v.end(), e, e + n);
+    }
+    std::sort(v.begin(), v.end(), [](const FctKernels &a, const FctKernels &b) {
+      return a.e.bluestein != b.e.bluestein ? a.e.bluestein < b.e.bluestein : a.e.len < b.e.len;
+    });
+    return v;
+  }();
+  return all;
+}
+
+// The FFT of one side: of n points if there is one, else the shortest that holds the
+// chirp convolution; null above the longest.
+const FctKernels *plan_side(int n, FctSide *d) {
+  d->n = n;
+  for (const FctKernels &k : lengths())
+    if (k.e.bluestein ? k.e.len >= 2 * n - 1 : k.e.len == n) {
+      d->bluestein = k.e.bluestein;
+      d->len = k.e.len;
+      return &k;
+    }
+  return nullptr;
+}
+
+size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// GDGS_DIRECT=0 keeps the multigrid cycles; so do the switches of the multigrid's
+// streaming passes (comparisons and tests name them).
+bool fct_enabled() {
+  static const bool on = [] {
+    const char *v = getenv("GDGS_DIRECT");
+    if (v) return v[0] != '0';
+    return !getenv("GDGS_STREAM") && !getenv("GDGS_STREAM_ROWS") && !getenv("GDGS_STREAM_UP_LEVELS") &&
+           !getenv("GDGS_STREAM_DOWN_LEVELS");
+  }();
+  return on;
+}
+
+// Opt the kernels of a length in to the shared memory their blocks take, once per device.
+cudaError_t opt_in(const FctKernels &k) {
+  static std::atomic<unsigned long long> done[160];
+  int dev = 0;
+  cudaError_t r = cudaGetDevice(&dev);
+  if (r != cudaSuccess) return r;
+  const size_t i = (size_t)(&k - lengths().data());
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (i < 160 && (done[i].load(std::memory_order_acquire) & bit)) return cudaSuccess;
+  const std::pair<FctKernel, int> need[4] = {
+      {k.rows, k.e.row_smem}, {k.cols, k.e.col_smem}, {k.back, k.e.row_smem}, {k.chirp, k.e.chirp_smem}};
+  for (const auto &n : need)
+    if (n.first && n.second > 48 * 1024 && r == cudaSuccess)
+      r = cudaFuncSetAttribute((const void *)n.first, cudaFuncAttributeMaxDynamicSharedMemorySize, n.second);
+  if (r == cudaSuccess && i < 160) done[i].fetch_or(bit, std::memory_order_acq_rel);
+  return r;
+}
+
+}  // namespace
+
+// The direct solve takes the default cycle options: a caller who sets the sweeps, the
+// relaxation or the coarsest grid gets the multigrid cycles he describes (they change
+// the way to the solution, not the solution). Sides up to the longest FFT length, 4096
+// points (Bluestein's convolution of 8192 points included).
+bool fct_plan(const PoissonArgs &a, FctPlan *f) {
+  if (a.nu1 != 2 || a.nu2 != 1 || a.omega != 1.2f || a.coarse_max_dim != 8 || !fct_enabled()) return false;
+  if (a.H < 2 || a.W < 2) return false;
+  f->ex = plan_side(a.W, &f->x);
+  f->ey = plan_side(a.H, &f->y);
+  if (!f->ex || !f->ey) return false;
+  f->cycles = std::min(a.max_cycles, kFctMaxCycles);
+  f->wp = (a.W + 7) & ~7;
+  // the arrays of the multigrid corrections and residuals, which this path does not use
+  const Plan &p = *a.plan;
+  size_t o = p.off_e0;
+  f->spec = (float *)(a.ws + o);
+  o = up256(o + sizeof(float) * (size_t)a.C * a.H * f->wp);
+  FctSide *sides[2] = {&f->x, &f->y};
+  for (FctSide *d : sides) {
+    d->tw = (float2 *)(a.ws + o);
+    o = up256(o + sizeof(float2) * (size_t)d->len);
+    d->th = (float2 *)(a.ws + o);
+    o = up256(o + sizeof(float2) * (size_t)d->n);
+    d->s2 = (float *)(a.ws + o);
+    o = up256(o + sizeof(float) * (size_t)d->n);
+    if (d->bluestein) {
+      d->chirp = (float2 *)(a.ws + o);
+      o = up256(o + sizeof(float2) * (size_t)d->n);
+      d->bhat = (float2 *)(a.ws + o);
+      o = up256(o + sizeof(float2) * (size_t)d->len);
+    }
+  }
+  return o <= p.total;
+}
+
+cudaError_t run_fct(const PoissonArgs &a, const FctPlan &f, const float *rho, float *uhi, float *ulo,
+                    cudaStream_t st) {
+  FctArgs fa{};
+  fa.x = f.x;
+  fa.y = f.y;
+  fa.C = a.C;
+  fa.H = a.H;
+  fa.W = a.W;
+  fa.wp = f.wp;
+  fa.rho = rho;
+  fa.uhi = uhi;
+  fa.ulo = ulo;
+  fa.spec = f.spec;
+  fa.image = a.image;
+  fa.inv_cells = 1.0 / ((double)a.H * a.W);
+  for (int c = 0; c < GDGS_MAX_CHANNELS; ++c) fa.mean[c] = a.mean[c];
+  fa.ctrl = a.ctrl;
+  cudaError_t e = opt_in(*f.ex);
+  if (e == cudaSuccess) e = opt_in(*f.ey);
+  if (e != cudaSuccess) return e;
+  const FctEntry &ex = f.ex->e, &ey = f.ey->e;
+  for (int i = 0; i < 2; ++i) {
+    const FctKernels &k = i ? *f.ey : *f.ex;
+    if (!k.e.bluestein) continue;
+    LaunchScope ls_("fct_chirp", st);
+    launch_k(k.chirp, 1, k.e.chirp_threads, k.e.chirp_smem, st, fa, i);
+  }
+  const dim3 rg(((a.H + 1) / 2 + ex.row_g - 1) / ex.row_g, a.C), cg(((a.W + 1) / 2 + ey.col_g - 1) / ey.col_g, a.C);
+  const int V = a.W % 4 == 0 ? 4 : 1;
+  const long long nq = (long long)a.H * (a.W / V);
+  const dim3 fg((unsigned)std::max<long long>(1, std::min<long long>((nq + 255) / 256, 608)), a.C);
+  for (int k = 0; k < f.cycles; ++k) {
+    {
+      LaunchScope ls_("mg0_down", st);
+      launch_k(f.ex->rows, rg, ex.row_threads, ex.row_smem, st, fa, k);
+    }
+    {
+      LaunchScope ls_("fct_columns", st);
+      launch_k(f.ey->cols, cg, ey.col_threads, ey.col_smem, st, fa, k);
+    }
+    {
+      LaunchScope ls_("mg0_up", st);
+      launch_k(f.ex->back, rg, ex.row_threads, ex.row_smem, st, fa, k);
+    }
+    if (k > 0 || f.cycles == 1) {
+      const int first = k == std::min(1, f.cycles - 1);
+      LaunchScope ls_("finalize", st);
+      if (V == 4) launch_k(fct_finalize_kernel<4>, fg, 256, 0, st, fa, k + 1, first);
+      else launch_k(fct_finalize_kernel<1>, fg, 256, 0, st, fa, k + 1, first);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace gdgs

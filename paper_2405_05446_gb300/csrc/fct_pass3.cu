@@ -1,0 +1,4 @@
+// FFT lengths of the direct solve, part 3 of 16 (fct_pass.cuh).
+#include "fct_pass.cuh"
+
+GDGS_FCT_SLICE(3)

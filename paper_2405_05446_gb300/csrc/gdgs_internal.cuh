@@ -35,7 +35,7 @@ struct Ctrl {
   int max_cycles;
   int channels;
   int iter;            // cycle index when the cycle loop runs as a graph
-  int pad1;
+  int direct;          // direct solve (cosine transforms): refinement cycles launched, 0 otherwise
   double rtol;
   double rnorm2[kMaxCycles + 1];             // ||rho - L u_k||^2, k = 0..
   double sum_u[kMaxCycles + 1][GDGS_MAX_CHANNELS];  // sum of u_k per channel
@@ -50,6 +50,10 @@ struct Ctrl {
   int split;
   int kf_c[GDGS_MAX_CHANNELS];
 };
+
+// Direct solve: rnorm2[] holds each channel's ||residual||^2 after q = 1 .. cycles
+// cycles, and (q = 0, written by the finalize pass) ||rho - mean||^2.
+__host__ __device__ constexpr int fct_slot(int q, int c) { return 1 + GDGS_MAX_CHANNELS * q + c; }
 
 // Diagnostics hooks around every kernel launch (diag.cu).
 void diag_before(const char *name, cudaStream_t st);
@@ -334,6 +338,7 @@ struct PoissonArgs {
   float rtol;
   float omega;              // smoother over-relaxation
   int storage;              // GDGS_STORAGE_*: multigrid corrections and coarse right-hand sides
+  int coarse_max_dim;
   const Plan *plan;
   char *ws;
   Ctrl *ctrl;

@@ -19,6 +19,10 @@
 // zero-mean solution of L u = f), built once per grid shape by Gauss-Jordan on
 // the device and cached in the workspace under a tag.
 //
+// With the default cycle options and sides up to 4096 pixels the divergence is followed
+// by the direct solve of fct.cu; the cycles below serve the other sizes and a caller's own
+// sweeps, relaxation or coarsest grid.
+//
 // Iteration. The finest iterate u is a float-float pair (hi + lo): an FP32
 // image carries a representation error that alone gives a relative residual
 // ~1e-5 on 1080p scenes, above the 1e-6 target. Cycle k solves L e = r_k with an
@@ -62,7 +66,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include "gdgs_internal.cuh"
+#include "fct.cuh"
 
 namespace gdgs {
 
@@ -2228,7 +2232,25 @@ struct DivArgs {
   float *rho;
   float rtol;
   int max_cycles;
+  int direct;      // refinement cycles of a direct solve (0: multigrid)
+  FctSide tx, ty;   // its tables, filled by the blocks of one more grid row
 };
+
+// The part of the divergence kernels that is not per pixel: the solve's parameters, and
+// (blocks with blockIdx.y == C) the tables of a direct solve. True: the block is done.
+__device__ __forceinline__ bool divergence_prologue(const DivArgs &a, Ctrl *ctrl) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    ctrl->rtol = a.rtol;
+    ctrl->max_cycles = a.max_cycles;
+    ctrl->channels = a.C;
+    ctrl->direct = a.direct;
+  }
+  if ((int)blockIdx.y < a.C) return false;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, n = gridDim.x * blockDim.x;
+  fct_build_tables(a.tx, tid, n);
+  fct_build_tables(a.ty, tid, n);
+  return true;
+}
 
 __device__ __forceinline__ bool tile_on(const uint8_t *mask, int tiles_x, int i, int j) {
   return !mask || mask[(i / kTile) * tiles_x + (j / kTile)];
@@ -2239,11 +2261,7 @@ __device__ __forceinline__ bool tile_on(const uint8_t *mask, int tiles_x, int i,
 // Laplacian fields); then the hard threshold T of Eq. thresh when t > 0; ||rho||^2.
 __global__ void __launch_bounds__(256) divergence_kernel(DivArgs a, Ctrl *ctrl) {
   griddep_enter();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-    ctrl->rtol = a.rtol;
-    ctrl->max_cycles = a.max_cycles;
-    ctrl->channels = a.C;
-  }
+  if (divergence_prologue(a, ctrl)) return;
   const int c = blockIdx.y;
   const size_t plane = (size_t)a.H * a.W;
   const float *gxp = a.maps + (size_t)(a.input_is_rho ? c : 2 * c) * plane;
@@ -2288,11 +2306,7 @@ __device__ __forceinline__ float4 ld_f4(const float *p) {
 
 __global__ void __launch_bounds__(256) divergence4_kernel(DivArgs a, Ctrl *ctrl) {
   griddep_enter();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-    ctrl->rtol = a.rtol;
-    ctrl->max_cycles = a.max_cycles;
-    ctrl->channels = a.C;
-  }
+  if (divergence_prologue(a, ctrl)) return;
   const int c = blockIdx.y, W = a.W, H = a.H, Wq = W >> 2, nq = H * Wq;
   const size_t plane = (size_t)H * W;
   const float *gxp = a.maps + (size_t)(a.input_is_rho ? c : 2 * c) * plane;
@@ -3059,22 +3073,26 @@ cudaError_t run_poisson(const PoissonArgs &a, cudaStream_t st) {
   float *ulo = (float *)(ws + p.off_ulo);
   cudaError_t e;
 
+  FctPlan fct{};
+  const bool direct = fct_plan(a, &fct);
   DivArgs d{a.maps, a.mask, a.input_is_rho, a.threshold, a.C, a.H, a.W, a.tiles_x, rho, a.rtol,
-            a.max_cycles};
+            a.max_cycles, direct ? fct.cycles : 0, fct.x, fct.y};
+  const int rows = a.C + (direct ? 1 : 0);
   {
     const size_t plane = (size_t)a.H * a.W;
     if (quad_path(a.W, a.maps, rho)) {
       const int bx = pixel_blocks(plane / 4);
       LaunchScope ls_("divergence", st);
-      launch_k(divergence4_kernel, dim3(bx, a.C), 256, 0, st, d, ctrl);
+      launch_k(divergence4_kernel, dim3(bx, rows), 256, 0, st, d, ctrl);
     } else {
       int bx = (int)((plane + 255) / 256);
       if (bx > 4096) bx = 4096;
       LaunchScope ls_("divergence", st);
-      launch_k(divergence_kernel, dim3(bx, a.C), 256, 0, st, d, ctrl);
+      launch_k(divergence_kernel, dim3(bx, rows), 256, 0, st, d, ctrl);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
+  if (direct) return run_fct(a, fct, rho, uhi, ulo, st);
 
   // coarse factor (cached in the workspace)
   const LevelGeom &gcoarse = p.lv[p.levels - 1];
