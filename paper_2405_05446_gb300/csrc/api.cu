@@ -111,7 +111,7 @@ bool make_plan(int64_t n, int C, int W, int H, const gdgs_raster_opts &ro,
     p->off_blocksum = cv.take(8 * (size_t)((n + kBinBlock - 1) / kBinBlock + 2));
     p->off_gtiles = cv.take(4 * (size_t)n);
     p->off_maps = cv.take(4 * (size_t)C * 2 * W * H);
-    p->off_dsplat = cv.take(24 * (size_t)n);
+    p->off_dsplat = cv.take(48 * (size_t)n);
   }
   p->off_range = cv.take(8 * (size_t)p->T);
   p->off_active = cv.take(4 * (size_t)p->T);
@@ -540,7 +540,7 @@ int gdgs_render_view_backward(const gdgs_gaussians *g, const gdgs_camera *cam,
   const size_t n = (size_t)g->n, plane = (size_t)cam->width * cam->height;
   // gradients accumulate (atomics) or are written per Gaussian: clear first
   if (cudaMemsetAsync(grads->d_attr, 0, 4 * n * Q, st) != cudaSuccess ||
-      (n && cudaMemsetAsync(w + p.off_dsplat, 0, 24 * n, st) != cudaSuccess) ||
+      (n && cudaMemsetAsync(w + p.off_dsplat, 0, 48 * n, st) != cudaSuccess) ||
       cudaMemsetAsync(wa + pa.off_ctrl, 0, sizeof(Ctrl), st) != cudaSuccess)
     return GDGS_ERR_CUDA;
   // 1. d rho = the zero-mean solve of d image (L symmetric), into the forward
@@ -602,7 +602,7 @@ int gdgs_render_view_backward(const gdgs_gaussians *g, const gdgs_camera *cam,
   r.alpha_max = ro.alpha_max;
   r.t_min = ro.t_min;
   r.mbar = (const float *)(w + p.off_maps);
-  r.dsplat = (float *)(w + p.off_dsplat);
+  r.dsplat = (double *)(w + p.off_dsplat);
   r.dattr = grads->d_attr;
   r.ctrl = (Ctrl *)(w + p.off_ctrl);
   if ((e = launch_raster_backward(r, st)) != cudaSuccess) return to_status(e);
@@ -617,7 +617,7 @@ int gdgs_render_view_backward(const gdgs_gaussians *g, const gdgs_camera *cam,
   pb.fy = cam->fy;
   pb.dilation = ro.dilation;
   pb.exp_coef = ro.exp_coef;
-  pb.dsplat = (const float *)(w + p.off_dsplat);
+  pb.dsplat = (const double *)(w + p.off_dsplat);
   pb.d_mean = grads->d_mean;
   pb.d_scale = grads->d_scale;
   pb.d_quat = grads->d_quat;
