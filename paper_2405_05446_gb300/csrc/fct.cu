@@ -9,10 +9,10 @@
 // solves L e = r exactly up to FP32 rounding. One cycle is three passes over the image:
 //   rows      residual r of the current iterate, its DCT along x        -> spectrum
 //   columns   DCT along y, the division by lambda, inverse DCT along y  -> spectrum
-//   rows back inverse DCT along x, u += e (float-float)
+//   rows back inverse DCT along x: the correction e
 // FP32 rounding of e leaves a relative residual of ~1e-5 (it is the size of the image's
 // own FP32 representation error), and the next cycle solves for exactly that: the
-// residual is evaluated from the float-float iterate with error-free sums, so two cycles
+// residual is evaluated without rounding errors that matter (fct_lap), so two cycles
 // reach ~1e-7 or less. The multigrid needs 4-6 cycles, each a chain of ~12 dependent
 // launches whose small levels leave the GPU idle (1080p, three channels: 150 us per
 // cycle, all latency); here every launch covers all channels and every SM.
@@ -68,7 +68,9 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
 #pragma unroll
     for (int i = 1; i < GDGS_MAX_CHANNELS; ++i)
       if (i == c) mc = a.mean[i];
-    s_shift = (float)((double)mc - a.ctrl->sum_u[s_kf][c] * a.inv_cells);
+    double sum = 0.0;  // of u: the sums of its corrections
+    for (int q = 1; q <= s_kf; ++q) sum += a.ctrl->sum_u[q][c];
+    s_shift = (float)((double)mc - sum * a.inv_cells);
     if (blockIdx.x == 0 && !s_skip) {
       a.ctrl->kf_c[c] = s_kf;
       a.ctrl->mean_set[c] = mc;
@@ -77,27 +79,23 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
   }
   __syncthreads();
   if (s_skip) return;
-  const FctMean mr = fct_block_mean(a, c);
+  const float mean_rho = fct_block_mean(a, c);
   const int kf = s_kf, W = a.W, H = a.H;
   const float shift = s_shift;
   const size_t plane = (size_t)H * W;
   const float *rho = a.rho + c * plane, *uh = a.uhi + c * plane, *ul = a.ulo + c * plane;
   float *img = a.image + c * plane;
   float r2 = 0.f;
-  const int Wq = W / V;
-  const long long nq = (long long)H * Wq;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < nq; q += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(q / Wq), j0 = (int)(q - (long long)i * Wq) * V;
-    const size_t p = (size_t)i * W + j0;
+  const int Wq = W / V, nq = H * Wq;  // H, W <= 4096
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
+    const int i = q / Wq, j0 = (q - i * Wq) * V, p = i * W + j0;
     if (kf == 0) {
 #pragma unroll
       for (int d = 0; d < V; ++d) img[p + d] = 0.f + (0.f + shift);
       continue;
     }
-    const size_t ps = i + 1 < H ? p + W : p, pn = i > 0 ? p - W : p;
-    float h[V + 2], l[V + 2], hs[V], ls[V], hn[V], ln[V], rv[V];
-    const bool low = kf > 1;
-    auto row = [&](const float *src, size_t o, float *dst) {
+    const int ps = i + 1 < H ? p + W : p, pn = i > 0 ? p - W : p;
+    auto row = [&](const float *src, int o, float *dst) {
       if constexpr (V == 4) {
         const float4 v = __ldg(reinterpret_cast<const float4 *>(src + o));
         dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w;
@@ -105,33 +103,29 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
         dst[0] = __ldg(src + o);
       }
     };
-    row(rho, p, rv);
-    row(uh, p, h + 1);
-    row(uh, ps, hs);
-    row(uh, pn, hn);
-    h[0] = j0 > 0 ? __ldg(uh + p - 1) : h[1];
-    h[V + 1] = j0 + V < W ? __ldg(uh + p + V) : h[V];
+    float r[V], h[V + 2], l[V + 2];
+    row(rho, p, r);
 #pragma unroll
-    for (int d = 0; d < V; ++d) l[d + 1] = ls[d] = ln[d] = 0.f;
-    l[0] = l[V + 1] = 0.f;
-    if (low) {
-      row(ul, p, l + 1);
-      row(ul, ps, ls);
-      row(ul, pn, ln);
-      l[0] = j0 > 0 ? __ldg(ul + p - 1) : l[1];
-      l[V + 1] = j0 + V < W ? __ldg(ul + p + V) : l[V];
-    }
+    for (int d = 0; d < V; ++d) l[d + 1] = 0.f;
+    // r -= L of one part of the iterate
+    auto minus_lap = [&](const float *u, float *c) {
+      float s[V], n[V];
+      row(u, p, c + 1);
+      row(u, ps, s);
+      row(u, pn, n);
+      c[0] = j0 > 0 ? __ldg(u + p - 1) : c[1];
+      c[V + 1] = j0 + V < W ? __ldg(u + p + V) : c[V];
+#pragma unroll
+      for (int d = 0; d < V; ++d) r[d] -= fct_lap(c[d + 1], c[d + 2], c[d], s[d], n[d]);
+    };
+    minus_lap(uh, h);
+    if (kf > 1) minus_lap(ul, l);
     float o[V];
-    FctDiff west = fct_diff<true>(h[1], l[1], h[0], l[0]);
 #pragma unroll
     for (int d = 0; d < V; ++d) {
-      const FctDiff east = fct_diff<true>(h[d + 2], l[d + 2], h[d + 1], l[d + 1]);
-      const FctDiff south = fct_diff<true>(hs[d], ls[d], h[d + 1], l[d + 1]);
-      const FctDiff north = fct_diff<true>(h[d + 1], l[d + 1], hn[d], ln[d]);
-      const float r = fct_residual(rv[d], mr.hi, mr.lo, east, west, south, north);
-      r2 = fmaf(r, r, r2);
+      r[d] -= mean_rho;
+      r2 = fmaf(r[d], r[d], r2);
       o[d] = h[d + 1] + (l[d + 1] + shift);
-      west = east;
     }
     if constexpr (V == 4) *reinterpret_cast<float4 *>(img + p) = make_float4(o[0], o[1], o[2], o[3]);
     else img[p] = o[0];

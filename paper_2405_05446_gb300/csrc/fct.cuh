@@ -143,64 +143,34 @@ __device__ __forceinline__ float fct_block_sum(float v) {
   return s;
 }
 
-// Error-free sums.
-__device__ __forceinline__ void fct_two_sum(float a, float b, float &s, float &e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+// The residual rho - mean - L u without rounding errors that matter, in plain FP32: the
+// first correction u_1 is stored rounded to multiples of one power of two g per channel,
+// about ulp(8 rms(u_1)) (fct_grid), so its differences and their sums are exact (below
+// 2^24 g; beyond, they round relative to themselves), and rho minus that sum loses nothing
+// where the two cancel. u can be 1e5 times as large as L u (smooth right-hand sides,
+// images spanning hundreds); with u_1 rounded to each value's own ulp the same sums were
+// off by more than the 1e-6 of rho that a cycle has to see, and error-free transformations
+// cost 70 instructions a pixel. The rounding itself is ~1e-6 of rms(u_1), like that of the
+// transforms, and goes into the next correction.
+__device__ __forceinline__ float fct_lap(float c, float e, float w, float s, float n) {
+  return __fadd_rn(__fadd_rn(__fsub_rn(e, c), __fsub_rn(w, c)), __fadd_rn(__fsub_rn(s, c), __fsub_rn(n, c)));
 }
 
-// The difference a - b of two neighbours u = h + l of the float-float iterate, as the
-// rounded difference of the high parts, its rounding error and (LOW: there are low parts)
-// the difference of the low parts.
-struct FctDiff {
-  float d, e;
-};
-template <bool LOW>
-__device__ __forceinline__ FctDiff fct_diff(float ah, float al, float bh, float bl) {
-  FctDiff r;
-  fct_two_sum(ah, -bh, r.d, r.e);
-  if (LOW) r.e += al - bl;
-  return r;
+// 3/2 2^23 g: adding and subtracting it rounds to multiples of g. sum2: the sum of squares
+// of u_1's scaled cosine coefficients, at most 4 of which make up the mean square of u_1.
+__device__ __forceinline__ float fct_grid(double sum2) {
+  const float rms8 = 16.f * sqrtf((float)sum2);
+  if (!(rms8 > 0.f) || !(rms8 < 1e37f)) return 0.f;
+  return 3.f * exp2f(ceilf(log2f(rms8)));
 }
+__host__ __device__ constexpr int fct_grid_slot(int c) { return fct_slot(kFctMaxCycles + 1, c); }
 
-// rho - mean - L u of one pixel from its differences to the east and south neighbours and
-// those of the west and north ones to it (0 where there is none). The sums are error-free:
-// u can be 1e5 times as large as L u (smooth right-hand sides, images spanning hundreds),
-// where a plain FP32 sum, or one without the errors of the differences at the zero
-// crossings of u, is off by more than the 1e-6 of rho a cycle has to see.
-__device__ __forceinline__ float fct_residual(float rho, float mh, float ml, FctDiff east, FctDiff west, FctDiff south,
-                                              FctDiff north) {
-  float s1, s2, s, f0, f1, f2, t, g;
-  fct_two_sum(east.d, -west.d, s1, f0);
-  fct_two_sum(south.d, -north.d, s2, f1);
-  fct_two_sum(s1, s2, s, f2);
-  const float err = ((f0 + f1) + f2) + ((east.e - west.e) + (south.e - north.e));
-  fct_two_sum(rho, -s, t, g);
-  return (t - mh) + ((g - err) - ml);
-}
-
-struct FctMean {
-  float hi, lo;
-};
-__device__ __forceinline__ FctMean fct_block_mean(const FctArgs &a, int c) {
-  __shared__ float s_m[2];
-  if (threadIdx.x == 0) {
-    const double m = a.ctrl->rho_sum[c] * a.inv_cells;
-    s_m[0] = (float)m;
-    s_m[1] = (float)(m - (double)(float)m);
-  }
+// The mean of rho over channel c.
+__device__ __forceinline__ float fct_block_mean(const FctArgs &a, int c) {
+  __shared__ float s_m;
+  if (threadIdx.x == 0) s_m = (float)(a.ctrl->rho_sum[c] * a.inv_cells);
   __syncthreads();
-  return {s_m[0], s_m[1]};
-}
-
-__device__ __forceinline__ void fct_ds_add(float &hi, float &lo, float e) {
-  float s, err;
-  fct_two_sum(hi, e, s, err);
-  const float l = __fadd_rn(lo, err);
-  const float h2 = __fadd_rn(s, l);
-  lo = __fsub_rn(l, __fsub_rn(h2, s));
-  hi = h2;
+  return s_m;
 }
 
 }  // namespace gdgs

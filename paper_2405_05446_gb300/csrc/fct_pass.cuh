@@ -233,10 +233,6 @@ template <int N>
 struct Num {
   static constexpr int value = N;
 };
-template <bool B>
-struct Flag {
-  static constexpr bool value = B;
-};
 
 // The inputs j, j + M, ... of a first-stage butterfly from f(i).
 template <int M, int R, class Fn>
@@ -320,13 +316,12 @@ struct Fft {
   static constexpr int STAGES = 2 + (R3 > 1) + (R4 > 1);
   static constexpr int TP = cmax(cmax(stage_threads(LEN, R1), stage_threads(LEN, R2)),
                                  cmax(stage_threads(LEN, R3), stage_threads(LEN, R4)));
-  // transforms per block: rows about 256 threads; columns a power of two of pairs, four
-  // (whole 32-byte sectors of a spectrum row) where a block holds them
+  // transforms per block: rows about 256 threads (128 and 512 were 1-6 % slower); columns
+  // the power of two of pairs that gives at most 384 threads (256 or 768: 5-40 % slower)
   static constexpr int G_ROWS = cmax(1, 256 / TP);
   static constexpr int cols_g() {
     int g = 1;
     while (g < 32 && 2 * g * TP <= 384) g *= 2;
-    while (g < 4 && 2 * g * TP <= kFctMaxThreads) g *= 2;
     return g;
   }
   static constexpr int G_COLS = cols_g();
@@ -468,12 +463,15 @@ __device__ __forceinline__ void dft(float2 *S, const FctSide &d, int t, bool sme
   }
 }
 
-constexpr int blocks_at_80_regs(int threads) { return cmax(1, 65536 / (80 * ceil_div(threads, 32) * 32)); }
+// Blocks per SM the register budget is set for: the passes wait for loads, barriers and
+// twiddles more than they issue, so more warps pay. Measured at 3840x2160x3, rows + columns + rows
+// back of a solve: 56 registers 652 us, 64 670 us, 80 704 us, 48 655 us (and slower at 1080p).
+constexpr int blocks_per_sm(int threads) { return cmax(1, 65536 / (56 * ceil_div(threads, 32) * 32)); }
 
 // Rows forward (kc: cycle; cycle 0 transforms rho, later ones the residual of the
 // iterate, whose norm cycle 1 records).
 template <class F, bool BL>
-__global__ void __launch_bounds__(ceil_div(F::G_ROWS * F::TP, 32) * 32, blocks_at_80_regs(F::G_ROWS * F::TP))
+__global__ void __launch_bounds__(ceil_div(F::G_ROWS * F::TP, 32) * 32, blocks_per_sm(F::G_ROWS * F::TP))
 fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
   griddep_enter();
   extern __shared__ float2 fct_sm[];
@@ -491,10 +489,17 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
   const float *rho = a.rho + c * plane;
   float acc = 0.f;
   if (kc > 0) {
-    const FctMean mr = fct_block_mean(a, c);
+    const float mean_rho = fct_block_mean(a, c);
     const float *uh = a.uhi + c * plane, *ul = a.ulo + c * plane;
-    auto residual_pairs = [&](auto low) {
-      constexpr bool LOW = decltype(low)::value;
+    // residual of columns j, j + 1 of both rows: the field given minus L of the part u
+    auto minus_lap = [&](const float *u, int j, float2 &ra, float2 &rb) {
+      const Patch h = ld_patch(u, ia, j, W, H);
+      ra.x -= fct_lap(h.a.x, h.a.y, h.al, h.b.x, h.n.x);
+      ra.y -= fct_lap(h.a.y, h.ar, h.a.x, h.b.y, h.n.y);
+      rb.x -= fct_lap(h.b.x, h.b.y, h.bl, h.s.x, h.a.x);
+      rb.y -= fct_lap(h.b.y, h.br, h.b.x, h.s.y, h.a.y);
+    };
+    if (t < TP) {
 #pragma unroll 2
       for (int m = t; m < (W + 1) / 2; m += TP) {
         const int j = 2 * m;
@@ -502,22 +507,10 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
         if (va) {
           ra = ld_pair(rho + (size_t)ia * W, j, W);
           if (vb) rb = ld_pair(rho + (size_t)(ia + 1) * W, j, W);
-          const Patch h = ld_patch(uh, ia, j, W, H);
-          Patch l{};
-          if (LOW) l = ld_patch(ul, ia, j, W, H);
-          // differences between neighbours, each used on both its sides
-          const FctDiff a0 = fct_diff<LOW>(h.a.x, l.a.x, h.al, l.al), a1 = fct_diff<LOW>(h.a.y, l.a.y, h.a.x, l.a.x),
-                        a2 = fct_diff<LOW>(h.ar, l.ar, h.a.y, l.a.y);
-          const FctDiff x0 = fct_diff<LOW>(h.a.x, l.a.x, h.n.x, l.n.x), x1 = fct_diff<LOW>(h.b.x, l.b.x, h.a.x, l.a.x);
-          const FctDiff y0 = fct_diff<LOW>(h.a.y, l.a.y, h.n.y, l.n.y), y1 = fct_diff<LOW>(h.b.y, l.b.y, h.a.y, l.a.y);
-          ra.x = fct_residual(ra.x, mr.hi, mr.lo, a1, a0, x1, x0);
-          ra.y = fct_residual(ra.y, mr.hi, mr.lo, a2, a1, y1, y0);
-          if (vb) {
-            const FctDiff b0 = fct_diff<LOW>(h.b.x, l.b.x, h.bl, l.bl), b1 = fct_diff<LOW>(h.b.y, l.b.y, h.b.x, l.b.x),
-                          b2 = fct_diff<LOW>(h.br, l.br, h.b.y, l.b.y);
-            rb.x = fct_residual(rb.x, mr.hi, mr.lo, b1, b0, fct_diff<LOW>(h.s.x, l.s.x, h.b.x, l.b.x), x1);
-            rb.y = fct_residual(rb.y, mr.hi, mr.lo, b2, b1, fct_diff<LOW>(h.s.y, l.s.y, h.b.y, l.b.y), y1);
-          }
+          minus_lap(uh, j, ra, rb);
+          if (kc > 1) minus_lap(ul, j, ra, rb);
+          ra = make_float2(ra.x - mean_rho, ra.y - mean_rho);
+          rb = vb ? make_float2(rb.x - mean_rho, rb.y - mean_rho) : make_float2(0.f, 0.f);
           acc = fmaf(ra.x, ra.x, acc);
           acc = fmaf(rb.x, rb.x, acc);
           if (j + 1 < W) {
@@ -528,10 +521,6 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
         S[m] = make_float2(ra.x, rb.x);
         if (j + 1 < W) S[W - 1 - m] = make_float2(ra.y, rb.y);
       }
-    };
-    if (t < TP) {
-      if (kc == 1) residual_pairs(Flag<false>{});
-      else residual_pairs(Flag<true>{});
     }
     __syncthreads();
   }
@@ -576,7 +565,7 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
 
 // Columns: DCT along y of G column pairs, the division by lambda, and back.
 template <class F, bool BL>
-__global__ void __launch_bounds__(ceil_div(F::G_COLS * F::TP, 32) * 32, blocks_at_80_regs(F::G_COLS * F::TP))
+__global__ void __launch_bounds__(ceil_div(F::G_COLS * F::TP, 32) * 32, blocks_per_sm(F::G_COLS * F::TP))
 fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
   griddep_enter();
   extern __shared__ float2 fct_sm[];
@@ -607,7 +596,9 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
     }
     if (in) *reinterpret_cast<float2 *>(col + (size_t)row_of(i) * wp) = make_float2(v.y, v.x);
   };
-  // the spectral step on points k and H - k of both columns
+  // the spectral step on points k and H - k of both columns (and, in the first cycle, the
+  // sum of squares that sets the grid of the iterate)
+  float acc = 0.f;
   auto spectral = [&] {
     if (t < TP) {
       const float lxa = in ? __ldg(a.x.s2 + ja) : 1.f, lxb = ja + 1 < W ? __ldg(a.x.s2 + ja + 1) : 1.f;
@@ -626,6 +617,8 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
         q.bk = q.bk * __fdividef(scale, lk + lxb);
         q.an = k == 0 ? 0.f : q.an * __fdividef(scale, ln + lxa);
         q.bn = k == 0 ? 0.f : q.bn * __fdividef(scale, ln + lxb);
+        if (in) acc = fmaf(q.ak, q.ak, fmaf(q.an, q.an, acc));
+        if (ja + 1 < W) acc = fmaf(q.bk, q.bk, fmaf(q.bn, q.bn, acc));
         dct_pre(q, tk, z, zn);
         S[k * G] = z;
         if (kn != k) S[kn * G] = zn;
@@ -654,11 +647,16 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
     if (t < TP)
       for (int i = t; i < H; i += TP) to_image(i, S[i * G]);
   }
+  if (kc == 0) {
+    acc = fct_block_sum(acc);
+    if (threadIdx.x == 0) atomicAdd(&a.ctrl->rnorm2[fct_grid_slot(c)], (double)acc);
+  }
 }
 
-// Rows back: e of G row pairs, u += e in float-float (cycle 0: u = e, no low part yet).
+// Rows back: the correction e of G row pairs. The iterate is kept as two parts: the first
+// correction (rounded to the channel's grid) and the sum of the later ones, 1e-5 of it.
 template <class F, bool BL>
-__global__ void __launch_bounds__(ceil_div(F::G_ROWS * F::TP, 32) * 32, blocks_at_80_regs(F::G_ROWS * F::TP))
+__global__ void __launch_bounds__(ceil_div(F::G_ROWS * F::TP, 32) * 32, blocks_per_sm(F::G_ROWS * F::TP))
 fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
   griddep_enter();
   extern __shared__ float2 fct_sm[];
@@ -686,58 +684,33 @@ fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
   constexpr float inv_len = 1.f / (float)F::LEN;
   float acc = 0.f;
   if (va) {
-    // four column pairs of both rows at a time: their loads first
-    constexpr int U = 4;
     const int half = (W + 1) / 2;
-    auto update = [&](auto cycle) {
-      constexpr int K = decltype(cycle)::value;
-      float *rh[2] = {uh + (size_t)ia * W, uh + (size_t)(ia + 1) * W};
-      float *rl[2] = {ul + (size_t)ia * W, ul + (size_t)(ia + 1) * W};
-      const int rows = vb ? 2 : 1;
-      for (int m0 = t; m0 < half; m0 += U * TP) {
-        float2 h[U][2], l[U][2];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            const int m = m0 + u * TP;
-            const bool v = m < half && r < rows;
-            h[u][r] = l[u][r] = make_float2(0.f, 0.f);
-            if (K > 0 && v) h[u][r] = ld_pair(rh[r], 2 * m, W);
-            if (K > 1 && v) l[u][r] = ld_pair(rl[r], 2 * m, W);
-          }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int m = m0 + u * TP, j = 2 * m;
-          if (m >= half) break;
-          const bool two = j + 1 < W;
-          float2 z0 = S[m], z1 = two ? S[W - 1 - m] : z0;
-          if (BL) {
-            z0 = chirp_out(z0, __ldg(a.x.chirp + m), inv_len);
-            if (two) z1 = chirp_out(z1, __ldg(a.x.chirp + W - 1 - m), inv_len);
-          }
-          const float2 e[2] = {make_float2(z0.y, z1.y), make_float2(z0.x, z1.x)};
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            if (r >= rows) break;
-            float2 hi = h[u][r], lo = l[u][r];
-            if (K == 0) {
-              hi = e[r];
-            } else {
-              fct_ds_add(hi.x, lo.x, e[r].x);
-              fct_ds_add(hi.y, lo.y, e[r].y);
-              st_pair(rl[r], j, W, lo);
-            }
-            st_pair(rh[r], j, W, hi);
-            acc += hi.x + lo.x;
-            if (two) acc += hi.y + lo.y;
-          }
-        }
+    float *out = kc == 0 ? uh : ul;
+    const float grid = kc == 0 ? fct_grid(a.ctrl->rnorm2[fct_grid_slot(c)]) : 0.f;
+    for (int m = t; m < half; m += TP) {
+      const int j = 2 * m;
+      const bool two = j + 1 < W;
+      float2 z0 = S[m], z1 = two ? S[W - 1 - m] : z0;
+      if (BL) {
+        z0 = chirp_out(z0, __ldg(a.x.chirp + m), inv_len);
+        if (two) z1 = chirp_out(z1, __ldg(a.x.chirp + W - 1 - m), inv_len);
       }
-    };
-    if (kc == 0) update(Num<0>{});
-    else if (kc == 1) update(Num<1>{});
-    else update(Num<2>{});
+      const float2 e[2] = {make_float2(z0.y, z1.y), make_float2(z0.x, z1.x)};
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        if (r == 1 && !vb) break;
+        const size_t row = (size_t)(ia + r) * W;
+        float2 v = e[r];
+        if (kc == 0) v = make_float2(__fsub_rn(__fadd_rn(v.x, grid), grid), __fsub_rn(__fadd_rn(v.y, grid), grid));
+        acc += v.x;
+        if (two) acc += v.y;
+        if (kc > 1) {
+          const float2 l = ld_pair(ul + row, j, W);
+          v = make_float2(v.x + l.x, v.y + l.y);
+        }
+        st_pair(out + row, j, W, v);
+      }
+    }
   }
   acc = fct_block_sum(acc);
   if (threadIdx.x == 0) atomicAdd(&a.ctrl->sum_u[kc + 1][c], (double)acc);
