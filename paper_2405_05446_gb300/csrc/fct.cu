@@ -192,8 +192,9 @@ cudaError_t opt_in(const FctKernels &k) {
   if (i < 160 && (done[i].load(std::memory_order_acquire) & bit)) return cudaSuccess;
   const std::pair<FctKernel, int> need[4] = {
       {k.rows, k.e.row_smem}, {k.cols, k.e.col_smem}, {k.back, k.e.row_smem}, {k.chirp, k.e.chirp_smem}};
+  // whatever the size: the kernels' static shared memory counts towards the 48 KB as well
   for (const auto &n : need)
-    if (n.first && n.second > 48 * 1024 && r == cudaSuccess)
+    if (n.first && r == cudaSuccess)
       r = cudaFuncSetAttribute((const void *)n.first, cudaFuncAttributeMaxDynamicSharedMemorySize, n.second);
   if (r == cudaSuccess && i < 160) done[i].fetch_or(bit, std::memory_order_acq_rel);
   return r;
