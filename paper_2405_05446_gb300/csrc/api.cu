@@ -3,6 +3,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "gdgs_internal.cuh"
 
 namespace gdgs {
@@ -74,9 +76,6 @@ bool make_plan(int64_t n, int C, int W, int H, const gdgs_raster_opts &ro,
   const int64_t cap = n * (int64_t)ro.pairs_per_gaussian;
   if (cap > 0x7fffffffll) return false;
   p->pair_cap = (unsigned)cap;
-  const int64_t dblk = (n + kRadixBlockSmall - 1) / kRadixBlockSmall;  // depth sort
-  const int64_t pblk = (cap + kRadixBlock - 1) / kRadixBlock;           // pair sort
-  p->radix_blocks_max = (int)(dblk > pblk ? dblk : pblk);
 
   // multigrid levels: coarsen until both sides <= coarse_max_dim, at least 2 levels
   int levels = 1;
@@ -107,7 +106,8 @@ bool make_plan(int64_t n, int C, int W, int H, const gdgs_raster_opts &ro,
       p->off_pval[b] = cv.take(4 * (size_t)p->pair_cap);
     }
     p->off_dlo = cv.take(4 * (size_t)n);
-    p->off_hist = cv.take(4 * 256 * (size_t)(p->radix_blocks_max + 1));
+    p->off_hist = cv.take(4 * std::max(sort_state_words(n, kDepthTile), sort_state_words(cap, kPairTile)));
+    p->off_sort = cv.take(4 * kSortWords);
     p->off_blocksum = cv.take(8 * (size_t)((n + kBinBlock - 1) / kBinBlock + 2));
     p->off_gtiles = cv.take(4 * (size_t)n);
     p->off_maps = cv.take(4 * (size_t)C * 2 * W * H);
@@ -214,6 +214,7 @@ ProjectArgs project_args(const gdgs_gaussians *g, const gdgs_camera *cam,
   a.sconic = (float4 *)(ws + p.off_sconic);
   a.key = (uint32_t *)(ws + p.off_dkey[0]);  // sorted in place by the depth sort
   a.key_lo = (uint32_t *)(ws + p.off_dlo);
+  a.sort_scratch = (uint32_t *)(ws + p.off_sort);
   a.rect = (uint2 *)(ws + p.off_rect);
   a.ctrl = (Ctrl *)(ws + p.off_ctrl);
   return a;
@@ -231,24 +232,31 @@ cudaError_t raster_path(const gdgs_gaussians *g, const gdgs_camera *cam,
   pa.cam_dev = cam_dev;
   cudaError_t e = launch_project(pa, st);
   if (e != cudaSuccess) return e;
-  uint32_t *hist = (uint32_t *)(ws + p.off_hist);
+  uint32_t *state = (uint32_t *)(ws + p.off_hist), *scratch = (uint32_t *)(ws + p.off_sort);
   uint2 *range = (uint2 *)(ws + p.off_range);
   uint32_t *active = (uint32_t *)(ws + p.off_active);
   uint8_t *mk = mask ? mask : (uint8_t *)(ws + p.off_mask);
-  const uint32_t *pval_sorted = (const uint32_t *)(ws + p.off_pval[0]);
+  uint32_t *const pv[2] = {(uint32_t *)(ws + p.off_pval[0]), (uint32_t *)(ws + p.off_pval[1])};
   if (g->n > 0) {
     // 1. depth order of the Gaussians (float-float depth: lo digit, then hi bits)
-    uint32_t *dk0 = (uint32_t *)(ws + p.off_dkey[0]), *dv0 = (uint32_t *)(ws + p.off_dval[0]);
-    uint32_t *dk1 = (uint32_t *)(ws + p.off_dkey[1]), *dv1 = (uint32_t *)(ws + p.off_dval[1]);
-    const int dblocks = (int)((g->n + kRadixBlockSmall - 1) / kRadixBlockSmall);
-    bool alt = false;
-    e = radix_sort_pairs(dk0, dv0, dk1, dv1, true, (const uint32_t *)(ws + p.off_dlo), nullptr,
-                         (unsigned)g->n, 32, hist, kRadixItemsSmall, dblocks, &alt, st);
+    DepthSort ds{};
+    for (int b = 0; b < 2; ++b) {
+      ds.key[b] = (uint32_t *)(ws + p.off_dkey[b]);
+      ds.val[b] = (uint32_t *)(ws + p.off_dval[b]);
+    }
+    ds.key_lo = (const uint32_t *)(ws + p.off_dlo);
+    ds.n = (unsigned)g->n;
+    ds.state = state;
+    ds.scratch = {scratch, scratch + 2 * kSortPasses * 256};
+    ds.range = range;
+    ds.tile_mask = mk;
+    ds.T = p.T;
+    ds.ctrl = ctrl;
+    e = sort_depth(ds, st);
     if (e != cudaSuccess) return e;
-    const uint32_t *order = alt ? dv1 : dv0;
     // 2. emit (tile, Gaussian) pairs in depth order
     BinArgs b{};
-    b.order = order;
+    b.order = ds.val[1];
     b.rect = (const uint2 *)(ws + p.off_rect);
     b.smean = (const float4 *)(ws + p.off_smean);
     b.sconic = (const float4 *)(ws + p.off_sconic);
@@ -260,36 +268,40 @@ cudaError_t raster_path(const gdgs_gaussians *g, const gdgs_camera *cam,
     b.blocksum = (unsigned long long *)(ws + p.off_blocksum);
     b.tiles = (uint32_t *)(ws + p.off_gtiles);
     b.pkey = (uint32_t *)(ws + p.off_pkey[0]);
-    b.pval = (uint32_t *)(ws + p.off_pval[0]);
+    b.pval = pv[0];
+    b.bins = scratch + kSortPasses * 256;
+    b.sort_state = state;
     b.ctrl = ctrl;
     e = launch_emit_pairs(b, st);
     if (e != cudaSuccess) return e;
-    // 3. stable sort of the pairs by tile id
-    int tbits = 0;
-    while ((1 << tbits) < p.T) ++tbits;
-    uint32_t *pk0 = (uint32_t *)(ws + p.off_pkey[0]), *pv0 = (uint32_t *)(ws + p.off_pval[0]);
-    uint32_t *pk1 = (uint32_t *)(ws + p.off_pkey[1]), *pv1 = (uint32_t *)(ws + p.off_pval[1]);
-    alt = false;
-    const int pblocks = (int)(((int64_t)p.pair_cap + kRadixBlock - 1) / kRadixBlock);
-    e = radix_sort_pairs(pk0, pv0, pk1, pv1, false, nullptr, &ctrl->n_pairs, p.pair_cap, tbits,
-                         hist, kRadixItems, pblocks, &alt, st);
-    if (e != cudaSuccess) return e;
-    const uint32_t *pk_sorted = alt ? pk1 : pk0;
-    pval_sorted = alt ? pv1 : pv0;
-    // 4. tile ranges, mask and active list
-    e = launch_tile_ranges(pk_sorted, ctrl, p.pair_cap, p.T, range, active, mk, st);
+    // 3. stable sort of the pairs by tile id, leaving tile ranges, mask and active list
+    PairSort ps{};
+    for (int k = 0; k < 2; ++k) {
+      ps.key[k] = (uint32_t *)(ws + p.off_pkey[k]);
+      ps.val[k] = pv[k];
+    }
+    ps.n_dev = &ctrl->n_pairs;
+    ps.cap = p.pair_cap;
+    ps.T = p.T;
+    ps.state = state;
+    ps.scratch = {scratch + kSortPasses * 256, scratch + 2 * kSortPasses * 256 + 8};
+    ps.range = range;
+    ps.active = active;
+    ps.tile_mask = mk;
+    ps.ctrl = ctrl;
+    e = sort_pairs(ps, st);
     if (e != cudaSuccess) return e;
   } else {
     e = cudaMemsetAsync(range, 0, 8 * (size_t)p.T, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(mk, 0, (size_t)p.T, st);
     if (e != cudaSuccess) return e;
   }
-  // 5. composite
+  // 4. composite
   RasterArgs r{};
   r.smean = (const float4 *)(ws + p.off_smean);
   r.sconic = (const float4 *)(ws + p.off_sconic);
   r.grad = g->grad;
-  r.pval = pval_sorted;
+  r.pval = pv[pair_passes(p.T) & 1];
   r.range = range;
   r.active = active;
   r.use_active = (use_mask && g->n > 0) ? 1 : 0;
@@ -583,14 +595,11 @@ int gdgs_render_view_backward(const gdgs_gaussians *g, const gdgs_camera *cam,
   d.mbar = (float *)(w + p.off_maps);
   if ((e = launch_divergence_adjoint(d, st)) != cudaSuccess) return to_status(e);
   // 3. the composite, tile by tile, back to front
-  int tbits = 0;
-  while ((1 << tbits) < p.T) ++tbits;
-  const bool alt = ((tbits + 7) / 8) % 2 == 1;  // the pair sort's passes swap buffers
   RasterBwdArgs r{};
   r.smean = (const float4 *)(w + p.off_smean);
   r.sconic = (const float4 *)(w + p.off_sconic);
   r.attr = g->grad;
-  r.pval = (const uint32_t *)(w + p.off_pval[alt ? 1 : 0]);
+  r.pval = (const uint32_t *)(w + p.off_pval[pair_passes(p.T) & 1]);
   r.range = (const uint2 *)(w + p.off_range);
   r.active = (const uint32_t *)(w + p.off_active);
   r.Q = Q;

@@ -13,11 +13,15 @@ namespace gdgs {
 constexpr int kTile = GDGS_TILE;        // raster tile edge (pixels)
 constexpr int kMaxCycles = 64;          // bound on V-cycles per solve
 constexpr int kMaxLevels = 24;          // bound on multigrid levels
-constexpr int kRadixThreads = 256;
-constexpr int kRadixItems = 8;          // keys per thread per radix block (pair sort)
-constexpr int kRadixBlock = kRadixThreads * kRadixItems;
-constexpr int kRadixItemsSmall = 2;     // depth sort (fewer keys): more, shorter blocks
-constexpr int kRadixBlockSmall = kRadixThreads * kRadixItemsSmall;
+// Radix sorts (sort.cu): threads and keys per thread of a pass's tiles; threads
+// per SM (four blocks of 64 registers); the histogram's threads; grids of a few
+// resident blocks per SM (152).
+constexpr int kSortThreadsPerSm = 1024;
+constexpr int kDepthThreads = 256, kDepthItems = 8, kDepthTile = kDepthThreads * kDepthItems;
+constexpr int kPairThreads = 256, kPairItems = 10, kPairTile = kPairThreads * kPairItems;
+constexpr int kHistThreads = 512, kHistGrid = 304, kSortGrid = 1216, kEmitGrid = 912;
+constexpr int kSortPasses = 5;  // of the depth sort; the pair sort has at most 4
+constexpr int kSortWords = 2 * (kSortPasses * 256 + 8);  // both sorts' digit counts and tickets
 constexpr int kBinBlock = 256;  // Gaussians per block of the pair count and emission
 constexpr uint32_t kInvalidKey = 0xFFFFFFFFu;
 
@@ -126,13 +130,12 @@ struct Plan {
   int C, W, H;
   int tiles_x, tiles_y, T;
   unsigned pair_cap;
-  int radix_blocks_max;
   // offsets in bytes from the workspace base
   size_t off_ctrl;
   size_t off_smean, off_sconic, off_rect;              // projected splats [n]
   size_t off_dkey[2], off_dval[2];                     // depth sort [n]
   size_t off_dlo;                                      // depth sort secondary key [n]
-  size_t off_hist;                                     // radix histograms
+  size_t off_hist, off_sort;                           // sorts: status words; counts and tickets
   size_t off_blocksum;                                 // scan partials
   size_t off_gtiles;                                   // tiles per depth-ordered Gaussian
   size_t off_pkey[2], off_pval[2];                     // pairs [pair_cap]
@@ -173,6 +176,7 @@ struct ProjectArgs {
   float w2c[12];
   float fx, fy, cx, cy, znear;
   int W, H, tiles_x, tiles_y;
+  uint32_t *sort_scratch;      // kSortWords words, zeroed here for the sorts that follow
   const gdgs_camera *cam_dev;  // when set, w2c .. znear are read from it on the device
   float alpha_min, dilation, exp_coef;
   // outputs (workspace)
@@ -188,18 +192,79 @@ struct ProjectArgs {
 };
 cudaError_t launch_project(const ProjectArgs &a, cudaStream_t st);
 
-// Stable LSD radix sort of 32-bit keys with 32-bit values over bits
-// [0, nbits). n = min(*n_dev, cap) if n_dev else cap. vals_in == nullptr means
-// the values are the element indices. lo_keys (nullable): a secondary key whose
-// low 8 bits order elements with equal keys (one extra pass, run first).
-// Blocks of kRadixThreads * items keys (items kRadixItems or kRadixItemsSmall),
-// max_blocks of them at most; hist holds 256 * (max_blocks + 1) words. Returns
-// in *out_is_alt whether the result sits in the alternate buffers.
-cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
-                             uint32_t *vals_alt, bool implicit_vals, const uint32_t *lo_keys,
-                             const unsigned long long *n_dev, unsigned cap, int nbits,
-                             uint32_t *hist, int items, int max_blocks, bool *out_is_alt,
-                             cudaStream_t st);
+// Radix sorts of 32-bit keys with 32-bit values, stable (sort.cu). The scratch is zeroed by
+// the projection; `state` holds what the tiles of two successive passes publish.
+size_t sort_state_words(long long keys, int tile);
+struct SortState {
+  uint32_t *tile, *sum, *prefix;  // [tiles][256], [groups][256] twice
+};
+struct SortScratch {
+  uint32_t *bins;    // [kSortPasses][256]
+  unsigned *ticket;  // [kSortPasses]
+};
+
+enum { kSortPlain, kSortLow, kSortRanges };
+
+struct SortPass {
+  const uint32_t *keys_in, *vals_in, *keys_next;
+  uint32_t *keys_out, *vals_out;
+  const unsigned long long *n_dev;
+  unsigned cap;
+  int shift;
+  const uint32_t *bins;
+  unsigned *ticket;
+  SortState state, state_next;  // this pass's; the next one's, cleared here (tile null: none)
+  Ctrl *ctrl;
+  uint2 *range;
+  uint32_t *active;
+  uint8_t *tile_mask;
+};
+
+// The Gaussians by depth: the primary keys' 32 bits, ties by the low 8 bits of key_lo, then
+// by index; the indices in order end up in val[1]. Also clears the tile ranges and mask.
+struct DepthSort {
+  uint32_t *key[2], *val[2];
+  const uint32_t *key_lo;
+  unsigned n;
+  uint32_t *state;
+  SortScratch scratch;
+  uint2 *range;
+  uint8_t *tile_mask;
+  int T;
+  Ctrl *ctrl;
+};
+cudaError_t sort_depth(const DepthSort &s, cudaStream_t st);
+
+// The pairs by tile: the Gaussians in order end up in val[pair_passes(T) & 1], each tile's
+// pairs in range (tile_range), the tiles that have any in active (ctrl->n_active of them,
+// in any order) and as 1 in tile_mask.
+struct PairSort {
+  uint32_t *key[2], *val[2];
+  const unsigned long long *n_dev;
+  unsigned cap;
+  int T;
+  uint32_t *state;
+  SortScratch scratch;
+  uint2 *range;
+  uint32_t *active;
+  uint8_t *tile_mask;
+  Ctrl *ctrl;
+};
+cudaError_t sort_pairs(const PairSort &s, cudaStream_t st);
+
+inline int tile_bits(int T) {
+  int b = 1;
+  while ((1 << b) < T) ++b;
+  return b;
+}
+inline int pair_passes(int T) { return (tile_bits(T) + 7) / 8; }
+inline int pair_digit(int T) { return (tile_bits(T) + pair_passes(T) - 1) / pair_passes(T); }
+
+// A tile's pairs: the sort leaves (~start, end), zero where there are none.
+__device__ __forceinline__ uint2 tile_range(const uint2 *range, int tile) {
+  const uint2 r = range[tile];
+  return r.y ? make_uint2(~r.x, r.y) : make_uint2(0u, 0u);
+}
 
 struct BinArgs {
   const uint32_t *order;   // Gaussian indices in depth order [n]
@@ -212,13 +277,12 @@ struct BinArgs {
   unsigned long long *blocksum;  // [ceil(n / kBinBlock) + 1]
   uint32_t *tiles;         // [n] tiles each depth-ordered Gaussian reaches (count -> emit)
   uint32_t *pkey, *pval;   // emitted pairs
+  uint32_t *bins, *sort_state;  // the pair sort's digit counts and published words
   Ctrl *ctrl;
+  SortState state;         // set by launch_emit_pairs, with the sort's passes
+  int passes, digit;
 };
 cudaError_t launch_emit_pairs(const BinArgs &a, cudaStream_t st);
-
-cudaError_t launch_tile_ranges(const uint32_t *sorted_keys, Ctrl *ctrl, unsigned pair_cap,
-                               int T, uint2 *range, uint32_t *active, uint8_t *mask,
-                               cudaStream_t st);
 
 // A projected splat staged for the 16x16 tile whose origin is (x0, y0), as the
 // forward and the backward rasteriser both evaluate it (the backward replays

@@ -2256,6 +2256,8 @@ __device__ __forceinline__ bool tile_on(const uint8_t *mask, int tiles_x, int i,
   return !mask || mask[(i / kTile) * tiles_x + (j / kTile)];
 }
 
+constexpr int kDivSpan = 128;  // pixels of one row per warp and step of the scalar divergence
+
 // rho(i,j) = [j<W-1] gx(i,j) - [j>=1] gx(i,j-1) + [i<H-1] gy(i,j) - [i>=1] gy(i-1,j),
 // with gradients of tiles whose mask is 0 read as zero (or rho read directly for
 // Laplacian fields); then the hard threshold T of Eq. thresh when t > 0; ||rho||^2.
@@ -2266,25 +2268,43 @@ __global__ void __launch_bounds__(256) divergence_kernel(DivArgs a, Ctrl *ctrl) 
   const size_t plane = (size_t)a.H * a.W;
   const float *gxp = a.maps + (size_t)(a.input_is_rho ? c : 2 * c) * plane;
   const float *gyp = gxp + plane;
+  float *rp = a.rho + (size_t)c * plane;
   bool bad = false;
   float n2 = 0.f, s1 = 0.f;
-  for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < plane;
-       p += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(p / a.W), j = (int)(p - (size_t)i * a.W);
-    float r = 0.f;
-    if (a.input_is_rho) {
-      if (tile_on(a.mask, a.tiles_x, i, j)) r = gxp[p];
-    } else {
-      if (j + 1 < a.W && tile_on(a.mask, a.tiles_x, i, j)) r += gxp[p];
-      if (j >= 1 && tile_on(a.mask, a.tiles_x, i, j - 1)) r -= gxp[p - 1];
-      if (i + 1 < a.H && tile_on(a.mask, a.tiles_x, i, j)) r += gyp[p];
-      if (i >= 1 && tile_on(a.mask, a.tiles_x, i - 1, j)) r -= gyp[p - a.W];
+  // a warp takes 128 pixels of one row, a lane every 32nd of them: one division for four
+  // pixels (a 64-bit division per pixel made this 60 us at 1617x768x4, see kDivSpan)
+  const int spans = (a.W + kDivSpan - 1) / kDivSpan, units = a.H * spans, lane = threadIdx.x & 31;
+  for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < units; u += (gridDim.x * blockDim.x) >> 5) {
+    const int i = u / spans, j0 = (u - i * spans) * kDivSpan + lane;
+    const size_t row = (size_t)i * a.W;
+    float v[kDivSpan / 32];
+#pragma unroll
+    for (int k = 0; k < kDivSpan / 32; ++k) {
+      const int j = j0 + 32 * k;
+      float r = 0.f;
+      if (j < a.W) {
+        const bool on = tile_on(a.mask, a.tiles_x, i, j);
+        if (a.input_is_rho) {
+          if (on) r = gxp[row + j];
+        } else {
+          if (j + 1 < a.W && on) r += gxp[row + j];
+          if (j >= 1 && tile_on(a.mask, a.tiles_x, i, j - 1)) r -= gxp[row + j - 1];
+          if (i + 1 < a.H && on) r += gyp[row + j];
+          if (i >= 1 && tile_on(a.mask, a.tiles_x, i - 1, j)) r -= gyp[row - a.W + j];
+        }
+      }
+      v[k] = r;
     }
-    bad |= !isfinite(r);
-    if (a.threshold > 0.f && !(fabsf(r) >= a.threshold)) r = 0.f;
-    a.rho[(size_t)c * plane + p] = r;
-    n2 = fmaf(r, r, n2);
-    s1 += r;
+#pragma unroll
+    for (int k = 0; k < kDivSpan / 32; ++k) {
+      const int j = j0 + 32 * k;
+      float r = v[k];
+      bad |= !isfinite(r);
+      if (a.threshold > 0.f && !(fabsf(r) >= a.threshold)) r = 0.f;
+      if (j < a.W) rp[row + j] = r;
+      n2 = fmaf(r, r, n2);
+      s1 += r;
+    }
   }
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) set_status(ctrl, GDGS_ERR_NONFINITE);
   n2 = block_sum(n2);
@@ -3085,8 +3105,7 @@ cudaError_t run_poisson(const PoissonArgs &a, cudaStream_t st) {
       LaunchScope ls_("divergence", st);
       launch_k(divergence4_kernel, dim3(bx, rows), 256, 0, st, d, ctrl);
     } else {
-      int bx = (int)((plane + 255) / 256);
-      if (bx > 4096) bx = 4096;
+      const int bx = pixel_blocks((size_t)a.H * ((a.W + kDivSpan - 1) / kDivSpan) * 32);  // 8 units per block
       LaunchScope ls_("divergence", st);
       launch_k(divergence_kernel, dim3(bx, rows), 256, 0, st, d, ctrl);
     }

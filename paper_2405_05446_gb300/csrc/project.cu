@@ -85,6 +85,8 @@ __device__ __forceinline__ uint32_t depth_lo_digit(FF t) {
 
 __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   griddep_enter();
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < kSortWords; t += gridDim.x * blockDim.x)
+    a.sort_scratch[t] = 0u;
   if (a.cam_dev) {  // camera from device memory (a graph replays for any camera)
     const gdgs_camera *cd = a.cam_dev;
 #pragma unroll

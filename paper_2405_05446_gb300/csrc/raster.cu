@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
   __shared__ float4 s_splat[kRasterThreads / 32][4 + QP][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned ntiles = a.use_active ? a.ctrl->n_active : (unsigned)a.T;
-  if (blockIdx.x >= ntiles) return;
+  if (blockIdx.x >= ntiles || a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // no sorted list
   const int tile = a.use_active ? (int)a.active[blockIdx.x] : (int)blockIdx.x;
   const int tyi = tile / a.tiles_x, txi = tile - tyi * a.tiles_x;
   const int x0 = txi * kTile, y0 = tyi * kTile;
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
   const bool in0 = px < a.W && py < a.H, in1 = px < a.W && py + 4 < a.H;
   const f32x2 fpx = pk(lx + 0.5f, lx + 0.5f), fpy = pk(ly + 0.5f, ly + 4.5f);
   const float x0f = (float)x0, y0f = (float)y0;
-  const uint2 rg = a.range[tile];
+  const uint2 rg = tile_range(a.range, tile);
   const float amin = a.alpha_min, amax = a.alpha_max, tmin = a.t_min;
   const f32x2 minus1 = pk(-1.f, -1.f);
   float4(*S)[32] = s_splat[warp];

@@ -14,12 +14,12 @@
 // Compared with a 64-bit (tile | depth) key this sorts 13 instead of 45 bits per
 // pair and moves 8 instead of 12 bytes per pair and pass.
 //
-// The radix sort is a classic LSD pass in three kernels (block histograms, one
-// scan over digit-major histograms, stable scatter, which also scans the 256
-// digit totals into the digit bases). Ranking inside a block is
-// stable: items are taken in rounds of 256 consecutive keys; within a warp peers
-// of a digit are found with __match_any_sync and ranked by lane; warps are
-// ranked in order through a shared-memory prefix per digit.
+// Each sort is one histogram kernel (the digit counts of every pass at once) and one
+// kernel per 8-bit pass that reads and writes every element once: a block ranks a tile of
+// keys, gets the counts of the tiles before it by looking back through their published
+// words (decoupled look-back: Merrill and Garland 2016; one pass per digit: Adinets and
+// Merrill 2022), reorders the tile in shared memory and writes runs of equal digits. The
+// last pass of the pair sort writes no keys: it leaves the tile ranges itself.
 #include <algorithm>
 
 #include "gdgs_internal.cuh"
@@ -40,29 +40,32 @@ __device__ __forceinline__ unsigned item_count(const unsigned long long *n_dev, 
   return n < cap ? (unsigned)n : cap;
 }
 
-template <int ITEMS>
-__global__ void __launch_bounds__(kRadixThreads)
-radix_hist_kernel(const uint32_t *keys, const unsigned long long *n_dev, unsigned cap,
-                  int shift, unsigned mask, uint32_t *hist) {
-  griddep_enter();
-  __shared__ unsigned sh[256];
-  const unsigned n = item_count(n_dev, cap);
-  const unsigned nb = (n + kRadixThreads * ITEMS - 1) / (kRadixThreads * ITEMS);
-  if (blockIdx.x >= nb) return;
-  sh[threadIdx.x] = 0;
-  __syncthreads();
-  const unsigned base = blockIdx.x * (kRadixThreads * ITEMS);
-#pragma unroll 4
-  for (int r = 0; r < ITEMS; ++r) {
-    const unsigned i = base + r * kRadixThreads + threadIdx.x;
-    if (i < n) atomicAdd(&sh[(keys[i] >> shift) & mask], 1u);
-  }
-  __syncthreads();
-  if (threadIdx.x <= mask) hist[threadIdx.x * nb + blockIdx.x] = sh[threadIdx.x];
+// Words that a pass's tiles leave for the tiles after them, one per digit:
+//   per tile        1 + the number of its keys (0: not there yet);
+//   per 16 tiles    the sum of their counts, and in the top bits how many of them it has;
+//   per 16 tiles    kPrefix | the keys of smaller digits and those of this digit in all tiles
+//                   up to the group's last (31 bits: there are at most 2^31 - 1 pairs).
+// A tile adds its own group's earlier tiles and then walks back group by group to the first
+// prefix. Walking back tile by tile instead read about 100 words a digit (several hundred
+// tiles are in flight): 140 us for a pass over 16.4M pairs.
+constexpr uint32_t kPrefix = 0x80000000u;
+constexpr int kGroup = 16, kGroupBits = 24;
+constexpr int kLookBack = 4;             // groups read at a time
+constexpr int kLookBackLimit = 1 << 19;  // polls before the wait gives up (about a second)
+
+__device__ __forceinline__ uint32_t ld_status(const uint32_t *p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
-// Block-wide exclusive scan of 32-bit values for 256 threads; *total = sum.
-__device__ __forceinline__ unsigned scan256(unsigned v, unsigned *total) {
+__device__ __forceinline__ void st_status(uint32_t *p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Exclusive scan of one value per digit, held by threads 0 .. 255 of a block.
+template <int THREADS>
+__device__ __forceinline__ unsigned scan_digits(unsigned v) {
   __shared__ unsigned wt[8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   unsigned x = v;
@@ -71,95 +74,244 @@ __device__ __forceinline__ unsigned scan256(unsigned v, unsigned *total) {
     const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) wt[w] = x;
+  if (lane == 31 && w < 8) wt[w] = x;
   __syncthreads();
-  unsigned before = 0, all = 0;
+  unsigned before = 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = 0; k < 7; ++k)
     if (k < w) before += wt[k];
-    all += wt[k];
-  }
-  __syncthreads();
-  *total = all;
   return x - v + before;
 }
 
-// Per digit d (one CTA each): exclusive scan of the block counts hist[d nb ..]
-// in place; the digit's total goes to tot[d].
-template <int ITEMS>
-__global__ void __launch_bounds__(256)
-radix_scan_digit_kernel(uint32_t *hist, uint32_t *tot, const unsigned long long *n_dev, unsigned cap) {
-  griddep_enter();
-  const unsigned n = item_count(n_dev, cap);
-  const unsigned nb = (n + kRadixThreads * ITEMS - 1) / (kRadixThreads * ITEMS);
-  uint32_t *h = hist + (size_t)blockIdx.x * nb;
-  unsigned run = 0;
-  for (unsigned base = 0; base < nb; base += 256) {
-    const unsigned i = base + threadIdx.x;
-    const unsigned v = i < nb ? h[i] : 0u;
-    unsigned t;
-    const unsigned ex = scan256(v, &t);
-    if (i < nb) h[i] = run + ex;
-    run += t;
-  }
-  if (threadIdx.x == 0) tot[blockIdx.x] = run;
+// Clears what the tiles of a pass publish, by threads tid of nt.
+__device__ __forceinline__ void clear_state(const SortState &s, unsigned tiles, unsigned tid, unsigned nt) {
+  const unsigned groups = (tiles + kGroup - 1) / kGroup;
+  for (unsigned t = tid; t < tiles * 256u; t += nt) s.tile[t] = 0u;
+  for (unsigned t = tid; t < groups * 256u; t += nt) s.sum[t] = s.prefix[t] = 0u;
 }
 
-// keys_next (nullable): the key written out for element i is keys_next[i]
-// instead of the key ranked on, so a first pass over a secondary key leaves the
-// primary keys in its order for the passes that follow. dtot: the digit totals;
-// every block scans them into the digit bases itself (256 values: cheaper than a
-// launch).
-template <int ITEMS>
-__global__ void __launch_bounds__(kRadixThreads)
-radix_scatter_kernel(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t *keys_out,
-                     uint32_t *vals_out, const unsigned long long *n_dev, unsigned cap, int shift,
-                     unsigned mask, const uint32_t *hist, const uint32_t *dtot,
-                     const uint32_t *keys_next) {
+// Digit counts of all passes of the depth sort (bins zeroed before), the cleared state of its
+// first pass, and the cleared tile ranges and mask of the pair sort that follows.
+__global__ void __launch_bounds__(kHistThreads) depth_hist_kernel(DepthSort a, SortState state) {
   griddep_enter();
-  constexpr int kWarps = kRadixThreads / 32;
-  __shared__ unsigned run[256];
-  __shared__ unsigned wcnt[kWarps][256];
-  const unsigned n = item_count(n_dev, cap);
-  const unsigned nb = (n + kRadixThreads * ITEMS - 1) / (kRadixThreads * ITEMS);
-  if (blockIdx.x >= nb) return;
-  const int w = threadIdx.x >> 5;
-  {
-    unsigned all;
-    const unsigned dbase = scan256(threadIdx.x <= mask ? dtot[threadIdx.x] : 0u, &all);
-    if (threadIdx.x <= mask) run[threadIdx.x] = dbase + hist[threadIdx.x * nb + blockIdx.x];
+  __shared__ unsigned sh[kSortPasses][256];
+  const unsigned tid = blockIdx.x * kHistThreads + threadIdx.x, nt = gridDim.x * kHistThreads;
+  for (int t = threadIdx.x; t < kSortPasses * 256; t += kHistThreads) (&sh[0][0])[t] = 0u;
+  clear_state(state, (a.n + kDepthTile - 1) / kDepthTile, tid, nt);
+  for (unsigned t = tid; t < (unsigned)a.T; t += nt) {
+    a.range[t] = make_uint2(0u, 0u);
+    a.tile_mask[t] = 0;
   }
-  const unsigned base = blockIdx.x * (kRadixThreads * ITEMS);
-  for (int r = 0; r < ITEMS; ++r) {
-    const unsigned i = base + r * kRadixThreads + threadIdx.x;
-    if (base + r * kRadixThreads >= n) break;  // uniform across the block
-    const bool valid = i < n;
-    const uint32_t key = valid ? keys_in[i] : 0u;
-    const uint32_t val = valid ? (vals_in ? vals_in[i] : i) : 0u;
-    const unsigned d = valid ? ((key >> shift) & mask) : 0x1000u;
-    for (int t = threadIdx.x; t < kWarps * 256; t += kRadixThreads) (&wcnt[0][0])[t] = 0u;
+  __syncthreads();
+  for (unsigned i = tid; i < a.n; i += nt) {
+    const uint32_t k = a.key[0][i];
+    atomicAdd(&sh[0][a.key_lo[i] & 255u], 1u);
+#pragma unroll
+    for (int p = 1; p < kSortPasses; ++p) atomicAdd(&sh[p][(k >> (8 * p - 8)) & 255u], 1u);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < kSortPasses * 256; t += kHistThreads) {
+    const unsigned c = (&sh[0][0])[t];
+    if (c) atomicAdd(&a.scratch.bins[t], c);
+  }
+}
+
+// One stable pass over 8 bits (or fewer) of the keys. Blocks draw tiles in order from a
+// ticket, so a tile waits only for tiles whose blocks already run; the waits are bounded.
+// What bounds it: the latency of a tile's chain (load, rank, look back, write) at half the
+// issue rate; the traffic is 16 bytes a pair, 40 us at 16.4M. Tiles of 2560 pairs with four
+// blocks an SM (64 registers without spills) were the fastest of 1536 .. 8192; ranking by
+// votes over the digit's bits (32 instructions) came out equal, __match_any_sync 20 % slower.
+// The seven passes of a 3840x2160 view (1M Gaussians, 16.4M pairs) 333 us, of 1920x1080 (200k,
+// 2.7M) 88 us, launch gaps included; block histogram, scan and scatter kernels for each pass
+// and a pass for the tile ranges took 735 and 196 us.
+// kKind: kSortPlain; kSortLow: ranked by the secondary keys, values are the indices and the
+// keys written are the primary ones; kSortRanges: the last pass over the pairs, whose output
+// is the values and each tile's range.
+template <int THREADS, int ITEMS, int BITS, int kKind>
+__global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pass_kernel(SortPass a) {
+  griddep_enter();
+  if (a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // an earlier pass gave up
+  constexpr int kWarps = THREADS / 32, kKeys = THREADS * ITEMS;
+  constexpr unsigned kMask = (1u << BITS) - 1u;
+  static_assert(THREADS >= 256 && THREADS % 32 == 0, "a thread per digit");
+  static_assert(ITEMS <= 32, "the list of run heads takes the counters' place, 16 bits a key");
+  extern __shared__ uint32_t sort_sm[];
+  uint32_t *const sk = sort_sm, *const sv = sk + kKeys;
+  uint2 *const wcnt = reinterpret_cast<uint2 *>(sv + kKeys);  // per warp and digit
+  __shared__ unsigned s_tile, s_heads, s_first[256], s_out[256];
+  const unsigned n = item_count(a.n_dev, a.cap), tiles = (n + kKeys - 1) / kKeys;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  uint2 *const row = wcnt + w * 256;
+  uint16_t *const head = reinterpret_cast<uint16_t *>(wcnt);
+  const unsigned lt = lanemask_lt();
+  if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
+  for (;;) {
+    for (int t = tid; t < kWarps * 256; t += THREADS) wcnt[t] = make_uint2(0u, 0u);
     __syncthreads();
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
-    const unsigned rank = __popc(peers & lanemask_lt());
-    if (valid && rank == 0) wcnt[w][d] = __popc(peers);
+    const unsigned tile = s_tile;
+    if (tile >= tiles) break;
+    const unsigned first = tile * (unsigned)kKeys, cnt = min(n - first, (unsigned)kKeys);
+    const unsigned group = tile / kGroup, member = tile % kGroup;
+    if (a.state_next.tile && tid < 256) {
+      a.state_next.tile[(size_t)tile * 256 + tid] = 0u;
+      if (member == 0) a.state_next.sum[group * 256 + tid] = a.state_next.prefix[group * 256 + tid] = 0u;
+    }
+    // a warp's keys are consecutive: index = (warp, item, lane)
+    const unsigned at = w * (32 * ITEMS) + lane;
+    uint32_t key[ITEMS];
+    unsigned pos[(ITEMS + 1) / 2] = {};  // two 16-bit ranks a word
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) key[r] = at + 32 * r < cnt ? a.keys_in[first + at + 32 * r] : 0u;
+    // rank among the warp's keys: the lanes of a digit meet in its word's mask
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const bool in = at + 32 * r < cnt;
+      uint2 *const slot = row + ((key[r] >> a.shift) & kMask);
+      if (in) atomicOr(&slot->y, 1u << lane);
+      __syncwarp();
+      const uint2 v = *slot;  // (keys of earlier items, lanes of this one)
+      const unsigned mine = __popc(v.y & lt);
+      __syncwarp();
+      if (in && mine == 0) *slot = make_uint2(v.x + __popc(v.y), 0u);
+      __syncwarp();
+      pos[r / 2] |= (v.x + mine) << (16 * (r & 1));
+    }
+    uint32_t val[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      if (kKind == kSortLow) val[r] = first + at + 32 * r;
+      else val[r] = at + 32 * r < cnt ? a.vals_in[first + at + 32 * r] : 0u;
+    }
     __syncthreads();
-    if (threadIdx.x <= mask) {
-      unsigned b2 = run[threadIdx.x];
+    unsigned c = 0;
+    if (tid < 256) {
 #pragma unroll
       for (int k = 0; k < kWarps; ++k) {
-        const unsigned c = wcnt[k][threadIdx.x];
-        wcnt[k][threadIdx.x] = b2;
-        b2 += c;
+        const unsigned x = wcnt[k * 256 + tid].x;
+        wcnt[k * 256 + tid].x = c;
+        c += x;
       }
-      run[threadIdx.x] = b2;
+      st_status(&a.state.tile[(size_t)tile * 256 + tid], 1u + c);
+      atomicAdd(&a.state.sum[group * 256 + tid], (1u << kGroupBits) + c);
     }
-    __syncthreads();
-    if (valid) {
-      const unsigned pos = wcnt[w][d] + rank;
-      keys_out[pos] = keys_next ? keys_next[i] : key;
-      vals_out[pos] = val;
+    const unsigned ex = scan_digits<THREADS>(c);
+    unsigned base = 0;
+    if (group == 0) {  // uniform: the first group starts at the digits' places
+      __syncthreads();
+      base = scan_digits<THREADS>(tid < 256 ? a.bins[tid] : 0u);
     }
+    if (tid < 256) s_first[tid] = ex;
     __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      if (at + 32 * r < cnt) {
+        const unsigned d = (key[r] >> a.shift) & kMask;
+        const unsigned q = s_first[d] + row[d].x + ((pos[r / 2] >> (16 * (r & 1))) & 0xffffu);
+        sk[q] = key[r];
+        sv[q] = val[r];
+      }
+    }
+    if (tid <= kMask) {
+      int polls = 0;
+      for (bool done = false; !done;) {  // the earlier tiles of the group
+        uint32_t s[kGroup - 1];
+#pragma unroll
+        for (int k = 0; k < kGroup - 1; ++k)
+          s[k] = k < (int)member ? ld_status(&a.state.tile[(size_t)(tile - 1 - k) * 256 + tid]) : 1u;
+        unsigned sum = 0;
+        done = true;
+#pragma unroll
+        for (int k = 0; k < kGroup - 1; ++k) {
+          done = done && s[k] != 0u;
+          sum += s[k] - 1u;
+        }
+        if (!done && ++polls > kLookBackLimit) {  // give up; the guard below keeps writes in bounds
+          set_status(a.ctrl, GDGS_ERR_TIMEOUT);
+          done = true;
+        }
+        if (done) base += sum;
+        else __nanosleep(64);
+      }
+      int g = (int)group - 1;
+      for (bool done = g < 0; !done;) {
+        uint32_t pre[kLookBack], sum[kLookBack];
+#pragma unroll
+        for (int k = 0; k < kLookBack; ++k) {
+          pre[k] = g - k >= 0 ? ld_status(&a.state.prefix[(g - k) * 256 + tid]) : 0u;
+          // (group 0: its prefix, which has the smaller digits' keys)
+          sum[k] = g - k > 0 ? ld_status(&a.state.sum[(g - k) * 256 + tid]) : 0u;
+        }
+        bool go = true;
+#pragma unroll
+        for (int k = 0; k < kLookBack; ++k) {
+          if (go && pre[k]) {
+            base += pre[k] & ~kPrefix;
+            done = true;
+          } else if (go && sum[k] >> kGroupBits == kGroup) {
+            base += sum[k] & ((1u << kGroupBits) - 1u);
+            --g;
+          } else {
+            go = false;
+          }
+          go = go && !done;
+        }
+        if (!done && ++polls > kLookBackLimit) {
+          set_status(a.ctrl, GDGS_ERR_TIMEOUT);
+          done = true;
+        }
+        if (!go && !done) __nanosleep(64);
+      }
+      if (member == kGroup - 1) st_status(&a.state.prefix[group * 256 + tid], kPrefix | ((base + c) & ~kPrefix));
+      s_out[tid] = base - ex;
+    }
+    if (kKind == kSortRanges && tid == 0) s_heads = 0;
+    __syncthreads();
+    if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
+#pragma unroll 4
+    for (int r = 0; r < ITEMS; ++r) {
+      const unsigned i = tid + r * THREADS;
+      if (i < cnt) {
+        const uint32_t k = sk[i], v = sv[i];
+        const unsigned q = s_out[(k >> a.shift) & kMask] + i;
+        if (q < n) {
+          a.vals_out[q] = v;
+          if (kKind == kSortPlain) a.keys_out[q] = k;
+          if (kKind == kSortLow) a.keys_out[q] = a.keys_next[v];
+          if (kKind == kSortRanges) {
+            // Runs of one tile are consecutive here (the earlier passes sorted the lower
+            // bits). Their ends go into the tile's range by a maximum, their heads are listed.
+            if (i + 1 == cnt || sk[i + 1] != k) atomicMax(&a.range[k].y, q + 1);
+            if (i == 0 || sk[i - 1] != k) head[atomicAdd(&s_heads, 1u)] = (uint16_t)i;
+          }
+        }
+      }
+    }
+    if (kKind == kSortRanges) {
+      // The heads: ~start by a maximum (0: none yet). The block that finds none lists the
+      // tile as active (in any order). All at once: an atomic's answer takes about 1 us.
+      __syncthreads();
+      const unsigned heads = s_heads;
+      for (unsigned h0 = w * 32; h0 < heads; h0 += THREADS) {
+        const unsigned h = h0 + lane;
+        uint32_t k = 0u;
+        bool fresh = false;
+        if (h < heads) {
+          const unsigned i = head[h];
+          k = sk[i];
+          fresh = atomicMax(&a.range[k].x, ~(s_out[(k >> a.shift) & kMask] + i)) == 0u;
+        }
+        const unsigned ball = __ballot_sync(0xffffffffu, fresh);
+        unsigned at0 = 0;
+        if (lane == 0 && ball) at0 = atomicAdd(&a.ctrl->n_active, __popc(ball));
+        at0 = __shfl_sync(0xffffffffu, at0, 0);
+        if (fresh) {
+          a.active[at0 + __popc(ball & lt)] = k;
+          a.tile_mask[k] = 1;
+        }
+      }
+      __syncthreads();  // before the counters are cleared for the next tile
+    }
   }
 }
 
@@ -274,7 +426,7 @@ __global__ void __launch_bounds__(kBinBlock) count_kernel(BinArgs a) {
   griddep_enter();
   const int64_t i = (int64_t)blockIdx.x * kBinBlock + threadIdx.x;
   unsigned long long s = 0;
-  if (i < a.n) {
+  if (i < a.n && a.ctrl->status != GDGS_ERR_TIMEOUT) {  // (then there is no order)
     const uint32_t g = a.order[i];
     const uint2 rc = a.rect[g];
     if (rect_tiles(rc)) s = tiles_hit(a, g, rc);
@@ -324,156 +476,218 @@ __global__ void __launch_bounds__(1024) blocksum_scan_kernel(BinArgs a, int nb) 
   }
 }
 
-// Pairs of one Gaussian per thread, at the offset its block's scan gives.
-__global__ void __launch_bounds__(kBinBlock) emit_kernel(BinArgs a) {
-  griddep_enter();
-  const int64_t i = (int64_t)blockIdx.x * kBinBlock + threadIdx.x;
-  const bool in = i < a.n;
-  uint32_t g = 0;
-  uint2 rc = make_uint2(0, 0);
-  unsigned cnt = 0u;
-  if (in) {
-    g = a.order[i];
-    rc = a.rect[g];
-    cnt = a.tiles[i];  // as counted by count_kernel
-  }
-  unsigned long long tot;
-  const unsigned long long my = a.blocksum[blockIdx.x] + block_exclusive_scan(cnt, &tot);
-  if (cnt) {
-    const Footprint f = footprint(a, g, rc);
-    unsigned long long p = my;
-    for (unsigned ty = f.y0; ty < f.y1; ++ty) {
-      unsigned lo, hi;
-      row_span(f, ty, &lo, &hi);
-      for (unsigned tx = lo; tx < hi; ++tx, ++p)
-        if (p < a.pair_cap) {
-          a.pkey[p] = ty * (unsigned)a.tiles_x + tx;
-          a.pval[p] = g;
-        }
-    }
-  }
+// The lane that holds element i, from the lanes' inclusive counts (31 beyond the last).
+__device__ __forceinline__ int owner(unsigned incl, unsigned i) {
+  int o = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1)
+    if (__shfl_sync(0xffffffffu, incl, o + step - 1) <= i) o += step;
+  return min(o, 31);
 }
 
-// Tile ranges from the boundaries in the tile-sorted keys, one pass over the
-// pairs: pair i starts its tile's run when key[i-1] differs and ends it when
-// key[i+1] differs. Ranges and mask are zeroed beforehand, so tiles without
-// pairs read (0, 0) and 0. A run's first pair also appends its tile to
-// `active` (order irrelevant: tiles are independent).
-__global__ void __launch_bounds__(256)
-ranges_kernel(const uint32_t *keys, Ctrl *ctrl, unsigned cap, uint2 *range, uint32_t *active,
-              uint8_t *mask) {
+// The pairs of kBinBlock depth-ordered Gaussians at a time, a warp's 32 in three steps: a
+// lane per Gaussian (its footprint, to shared memory), a lane per row of tiles (its span), a
+// lane per pair, so that the stores are whole lines (a thread per Gaussian wrote 32 scattered
+// words a store: 16.4M pairs 165 us and 62 us more for the digit counts, now 91 us). Also counts the pairs' digits for the sort and
+// clears what its first pass publishes.
+__global__ void __launch_bounds__(kBinBlock) emit_kernel(BinArgs a, int nb) {
   griddep_enter();
-  const unsigned long long np = ctrl->n_pairs;
-  const unsigned n = np < cap ? (unsigned)np : cap;
-  unsigned *rw = reinterpret_cast<unsigned *>(range);
-  const int lane = threadIdx.x & 31;
-  const unsigned stride = gridDim.x * blockDim.x;
-  for (unsigned i0 = blockIdx.x * blockDim.x; i0 < n; i0 += stride) {  // uniform per warp
-    const unsigned i = i0 + threadIdx.x;
-    const bool in = i < n;
-    const uint32_t k = in ? keys[i] : 0u;
-    const bool start = in && (i == 0 || keys[i - 1] != k);
-    const bool end = in && (i + 1 == n || keys[i + 1] != k);
-    if (start) {
-      rw[2 * (size_t)k] = i;
-      mask[k] = 1;
+  if (a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // no order
+  __shared__ Footprint s_f[kBinBlock];
+  __shared__ unsigned s_bins[4][256];
+  const int tid = threadIdx.x, lane = tid & 31, w0 = tid & ~31;
+  for (int t = tid; t < 4 * 256; t += kBinBlock) (&s_bins[0][0])[t] = 0u;
+  const unsigned np = item_count(&a.ctrl->n_pairs, a.pair_cap);
+  clear_state(a.state, (np + kPairTile - 1) / kPairTile, blockIdx.x * kBinBlock + tid, gridDim.x * kBinBlock);
+  const unsigned mask = (1u << a.digit) - 1u, full = 0xffffffffu;
+  for (int block = blockIdx.x; block < nb; block += gridDim.x) {
+    const int64_t i = (int64_t)block * kBinBlock + tid;
+    uint32_t g = 0;
+    unsigned cnt = 0u, rows = 0u;
+    if (i < a.n) {
+      g = a.order[i];
+      cnt = a.tiles[i];  // as counted by count_kernel
     }
-    if (end) rw[2 * (size_t)k + 1] = i + 1;
-    const unsigned ball = __ballot_sync(0xffffffffu, start);
-    unsigned base = 0;
-    if (lane == 0 && ball) base = atomicAdd(&ctrl->n_active, __popc(ball));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (start) active[base + __popc(ball & ((1u << lane) - 1u))] = k;
+    if (cnt) {
+      const Footprint f = footprint(a, g, a.rect[g]);
+      s_f[tid] = f;
+      rows = f.y1 - f.y0;
+    }
+    unsigned long long tot;  // (its barriers also order s_bins)
+    const unsigned long long my = a.blocksum[block] + block_exclusive_scan(cnt, &tot);
+    unsigned long long at = __shfl_sync(full, my, 0);  // where the warp's next pair goes
+    unsigned re = rows;  // rows of the warp's Gaussians up to this one
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(full, re, o);
+      if (lane >= o) re += y;
+    }
+    const unsigned nrows = __shfl_sync(full, re, 31);
+    for (unsigned r0 = 0; r0 < nrows; r0 += 32) {
+      const unsigned r = r0 + lane;
+      const int o = owner(re, r);
+      const unsigned before = __shfl_sync(full, re - rows, o);
+      const uint32_t rg = __shfl_sync(full, g, o);
+      unsigned len = 0, key0 = 0;
+      if (r < nrows) {
+        const Footprint &f = s_f[w0 + o];
+        const unsigned ty = f.y0 + (r - before);
+        unsigned lo, hi;
+        row_span(f, ty, &lo, &hi);
+        len = hi - lo;
+        key0 = ty * (unsigned)a.tiles_x + lo;
+      }
+      unsigned le = len;
+#pragma unroll
+      for (int k = 1; k < 32; k <<= 1) {
+        const unsigned y = __shfl_up_sync(full, le, k);
+        if (lane >= k) le += y;
+      }
+      const unsigned npairs = __shfl_sync(full, le, 31);
+      // digits above the first: a row of tiles has one or two of each
+      const unsigned long long p0 = at + (le - len);
+      const unsigned kept = p0 >= a.pair_cap ? 0u : (unsigned)min((unsigned long long)len, a.pair_cap - p0);
+      for (int p = 1; p < a.passes; ++p) {
+        const int shift = p * a.digit;
+        for (unsigned k = key0, end = key0 + kept; k < end;) {
+          const unsigned next = min(end, ((k >> shift) + 1u) << shift);
+          atomicAdd(&s_bins[p][(k >> shift) & mask], next - k);
+          k = next;
+        }
+      }
+      for (unsigned j0 = 0; j0 < npairs; j0 += 32) {
+        const unsigned j = j0 + lane;
+        const int q = owner(le, j);
+        const uint32_t key = __shfl_sync(full, key0 - (le - len), q) + j, val = __shfl_sync(full, rg, q);
+        const unsigned long long pos = at + j;
+        if (j < npairs && pos < a.pair_cap) {
+          a.pkey[pos] = key;
+          a.pval[pos] = val;
+          atomicAdd(&s_bins[0][key & mask], 1u);
+        }
+      }
+      at += npairs;
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < a.passes * 256; t += kBinBlock) {
+    const unsigned c = (&s_bins[0][0])[t];
+    if (c) atomicAdd(&a.bins[t], c);
   }
 }
 
 }  // namespace
 
-template <int ITEMS>
-cudaError_t radix_pass(const uint32_t *ki, const uint32_t *vi, uint32_t *ko, uint32_t *vo,
-                       const uint32_t *knext, const unsigned long long *n_dev, unsigned cap,
-                       int shift, unsigned mask, uint32_t *hist, unsigned blocks,
-                       cudaStream_t st) {
-  { LaunchScope ls_("radix_hist", st); launch_k(radix_hist_kernel<ITEMS>, blocks, kRadixThreads, 0, st, ki, n_dev, cap, shift, mask, hist); }
-  uint32_t *dtot = hist + (size_t)256 * blocks;
-  { LaunchScope ls_("radix_scan", st); launch_k(radix_scan_digit_kernel<ITEMS>, mask + 1, 256, 0, st, hist, dtot, n_dev, cap); }
+namespace {
+
+template <int THREADS, int ITEMS>
+constexpr int sort_smem() {
+  return 4 * (2 * THREADS * ITEMS + THREADS / 32 * 512);
+}
+
+template <int THREADS, int ITEMS, int BITS, int kKind>
+cudaError_t launch_pass(const SortPass &a, unsigned tiles, cudaStream_t st) {
+  constexpr int smem = sort_smem<THREADS, ITEMS>();
+  const auto kern = sort_pass_kernel<THREADS, ITEMS, BITS, kKind>;
+  static_assert(smem <= 40 * 1024, "with the static arrays within 48 KB");
+  LaunchScope ls_("radix_pass", st);
+  launch_k(kern, std::min<unsigned>(tiles, kSortGrid), THREADS, smem, st, a);
+  return cudaGetLastError();
+}
+
+template <int kKind>
+cudaError_t launch_pair_pass(const SortPass &a, int digit, unsigned tiles, cudaStream_t st) {
+  switch (digit) {
+    case 8: return launch_pass<kPairThreads, kPairItems, 8, kKind>(a, tiles, st);
+    case 7: return launch_pass<kPairThreads, kPairItems, 7, kKind>(a, tiles, st);
+    case 6: return launch_pass<kPairThreads, kPairItems, 6, kKind>(a, tiles, st);
+    default: return launch_pass<kPairThreads, kPairItems, 5, kKind>(a, tiles, st);
+  }
+}
+
+unsigned pair_tiles(unsigned cap) { return (unsigned)(((unsigned long long)cap + kPairTile - 1) / kPairTile); }
+
+// The words of one of two successive passes over at most `tiles` tiles.
+SortState sort_state(uint32_t *base, int which, unsigned tiles) {
+  const size_t groups = (tiles + kGroup - 1) / kGroup;
+  uint32_t *p = base + which * (size_t)256 * (tiles + 2 * groups);
+  return {p, p + (size_t)256 * tiles, p + (size_t)256 * (tiles + groups)};
+}
+
+}  // namespace
+
+size_t sort_state_words(long long keys, int tile) {
+  const size_t tiles = (size_t)((keys + tile - 1) / tile), groups = (tiles + kGroup - 1) / kGroup;
+  return 2 * 256 * (tiles + 2 * groups);
+}
+
+cudaError_t sort_depth(const DepthSort &s, cudaStream_t st) {
+  const unsigned tiles = (unsigned)((s.n + kDepthTile - 1) / kDepthTile);
+  if (tiles == 0) return cudaSuccess;
   {
-    LaunchScope ls_("radix_scatter", st);
-    launch_k(radix_scatter_kernel<ITEMS>, blocks, kRadixThreads, 0, st, ki, vi, ko, vo, n_dev, cap,
-             shift, mask, (const uint32_t *)hist, (const uint32_t *)dtot, knext);
+    LaunchScope ls_("radix_hist", st);
+    launch_k(depth_hist_kernel, std::min<unsigned>((s.n + 4 * kHistThreads - 1) / (4 * kHistThreads), kHistGrid),
+             kHistThreads, 0, st, s, sort_state(s.state, 0, tiles));
   }
-  return cudaGetLastError();
-}
-
-template <int ITEMS>
-cudaError_t radix_sort_t(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
-                         bool implicit_vals, const uint32_t *lo_keys,
-                         const unsigned long long *n_dev, unsigned cap, int nbits,
-                         uint32_t *hist, int max_blocks, bool *out_is_alt, cudaStream_t st) {
-  uint32_t *ki = keys, *vi = vals, *ko = keys_alt, *vo = vals_alt;
-  bool alt = false;
-  bool first = true;
-  const unsigned blocks = (unsigned)max_blocks;
-  if (blocks == 0) {
-    *out_is_alt = false;
-    return cudaSuccess;
-  }
-  if (lo_keys) {  // secondary key first (LSD): its low 8 bits, carrying the primary keys
-    cudaError_t e = radix_pass<ITEMS>(lo_keys, implicit_vals ? nullptr : vi, ko, vo, ki, n_dev,
-                                      cap, 0, 0xffu, hist, blocks, st);
+  for (int p = 0; p < kSortPasses; ++p) {
+    SortPass a{};
+    a.keys_in = p ? s.key[p & 1] : s.key_lo;
+    a.vals_in = s.val[p & 1];
+    a.keys_next = s.key[0];
+    a.keys_out = s.key[~p & 1];
+    a.vals_out = s.val[~p & 1];
+    a.cap = s.n;
+    a.shift = p ? 8 * (p - 1) : 0;
+    a.bins = s.scratch.bins + 256 * p;
+    a.ticket = s.scratch.ticket + p;
+    a.state = sort_state(s.state, p & 1, tiles);
+    if (p + 1 < kSortPasses) a.state_next = sort_state(s.state, ~p & 1, tiles);
+    a.ctrl = s.ctrl;
+    const cudaError_t e = p ? launch_pass<kDepthThreads, kDepthItems, 8, kSortPlain>(a, tiles, st)
+                            : launch_pass<kDepthThreads, kDepthItems, 8, kSortLow>(a, tiles, st);
     if (e != cudaSuccess) return e;
-    first = false;
-    uint32_t *t = ki; ki = ko; ko = t;
-    t = vi; vi = vo; vo = t;
-    alt = !alt;
   }
-  for (int shift = 0; shift < nbits; shift += 8) {
-    const int bits = nbits - shift < 8 ? nbits - shift : 8;
-    const unsigned mask = (1u << bits) - 1u;
-    cudaError_t e = radix_pass<ITEMS>(ki, (first && implicit_vals) ? nullptr : vi, ko, vo, nullptr,
-                                      n_dev, cap, shift, mask, hist, blocks, st);
+  return cudaSuccess;
+}
+
+cudaError_t sort_pairs(const PairSort &s, cudaStream_t st) {
+  const unsigned tiles = pair_tiles(s.cap);
+  if (tiles == 0) return cudaSuccess;
+  const int passes = pair_passes(s.T), digit = pair_digit(s.T);
+  for (int p = 0; p < passes; ++p) {
+    SortPass a{};
+    a.keys_in = s.key[p & 1];
+    a.vals_in = s.val[p & 1];
+    a.keys_out = s.key[~p & 1];
+    a.vals_out = s.val[~p & 1];
+    a.n_dev = s.n_dev;
+    a.cap = s.cap;
+    a.shift = p * digit;
+    a.bins = s.scratch.bins + 256 * p;
+    a.ticket = s.scratch.ticket + p;
+    a.state = sort_state(s.state, p & 1, tiles);
+    if (p + 1 < passes) a.state_next = sort_state(s.state, ~p & 1, tiles);
+    a.ctrl = s.ctrl;
+    a.range = s.range;
+    a.active = s.active;
+    a.tile_mask = s.tile_mask;
+    const cudaError_t e = p + 1 < passes ? launch_pair_pass<kSortPlain>(a, digit, tiles, st)
+                                         : launch_pair_pass<kSortRanges>(a, digit, tiles, st);
     if (e != cudaSuccess) return e;
-    first = false;
-    uint32_t *t = ki; ki = ko; ko = t;
-    t = vi; vi = vo; vo = t;
-    alt = !alt;
   }
-  *out_is_alt = alt;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
-cudaError_t radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt,
-                             uint32_t *vals_alt, bool implicit_vals, const uint32_t *lo_keys,
-                             const unsigned long long *n_dev, unsigned cap, int nbits,
-                             uint32_t *hist, int items, int max_blocks, bool *out_is_alt,
-                             cudaStream_t st) {
-  if (items == kRadixItemsSmall)
-    return radix_sort_t<kRadixItemsSmall>(keys, vals, keys_alt, vals_alt, implicit_vals, lo_keys,
-                                          n_dev, cap, nbits, hist, max_blocks, out_is_alt, st);
-  if (items == kRadixItems)
-    return radix_sort_t<kRadixItems>(keys, vals, keys_alt, vals_alt, implicit_vals, lo_keys, n_dev,
-                                     cap, nbits, hist, max_blocks, out_is_alt, st);
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_emit_pairs(const BinArgs &a, cudaStream_t st) {
-  if (a.n == 0) return cudaSuccess;
+cudaError_t launch_emit_pairs(const BinArgs &b, cudaStream_t st) {
+  if (b.n == 0) return cudaSuccess;
+  BinArgs a = b;
+  a.state = sort_state(b.sort_state, 0, pair_tiles(b.pair_cap));
+  a.passes = pair_passes(b.T);
+  a.digit = pair_digit(b.T);
   const int nb = (int)((a.n + kBinBlock - 1) / kBinBlock);
   { LaunchScope ls_("pair_count", st); launch_k(count_kernel, nb, kBinBlock, 0, st, a); }
   { LaunchScope ls_("pair_scan", st); launch_k(blocksum_scan_kernel, 1, 1024, 0, st, a, nb); }
-  { LaunchScope ls_("pair_emit", st); launch_k(emit_kernel, nb, kBinBlock, 0, st, a); }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_tile_ranges(const uint32_t *sorted_keys, Ctrl *ctrl, unsigned pair_cap,
-                               int T, uint2 *range, uint32_t *active, uint8_t *mask,
-                               cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(range, 0, 8 * (size_t)T, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(mask, 0, (size_t)T, st);
-  if (e != cudaSuccess) return e;
-  const unsigned blocks = (unsigned)std::min<unsigned long long>((pair_cap + 255ull) / 256, 2048);
-  if (blocks == 0) return cudaSuccess;
-  { LaunchScope ls_("tile_ranges", st); launch_k(ranges_kernel, blocks, 256, 0, st, sorted_keys, ctrl, pair_cap, range, active, mask); }
+  { LaunchScope ls_("pair_emit", st); launch_k(emit_kernel, std::min(nb, kEmitGrid), kBinBlock, 0, st, a, nb); }
   return cudaGetLastError();
 }
 
