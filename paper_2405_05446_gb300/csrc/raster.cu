@@ -43,8 +43,15 @@ namespace gdgs {
 namespace {
 
 constexpr int kRasterThreads = 128;
+// Up to 16 tiles per SM (152) the warps are too few to hide the three loads that follow one
+// another in a batch (index, splat, attribute), and the kernel loads ahead; above, the 8 to 34
+// registers that takes cost more than they give. Without and with: 243x143 with 294k Gaussians
+// 731 -> 534 us (144 tiles; a pixel per lane 659), 500x300 with 300k 348 -> 264 us (608 tiles),
+// 1237x711 with 300k 180 -> 178 us (3510), the 1080p view 489 -> 494 us (8160), the 2160p one
+// 1946 -> 2040 us (32400).
+constexpr int kAheadTiles = 2432;
 
-template <int Q>
+template <int Q, bool kAhead>
 __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
   griddep_enter();
   constexpr int QP = (Q + 1) / 2;  // 16-byte slots of the doubled attribute
@@ -73,41 +80,8 @@ __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
   for (int q = 0; q < Q; ++q) acc[q] = pk(0.f, 0.f);
   float T0 = in0 ? 1.f : 0.f, T1 = in1 ? 1.f : 0.f;  // 0: stopped (or outside)
 
-  for (unsigned s = rg.x; s < rg.y; s += 32) {
-    if (!__any_sync(0xffffffffu, T0 + T1 > 0.f)) break;
-    const unsigned j = s + lane;
-    StagedSplat st;
-    uint32_t g = 0;
-    bool in = false;
-    if (j < rg.y) {
-      g = a.pval[j];
-      const float4 kc = a.sconic[g];
-      st = stage_splat(a.smean[g], kc, x0f, y0f);
-      in = reaches_block<8>(st, kc, amin, by, bx);
-    }
-    const unsigned ball = __ballot_sync(0xffffffffu, in);
-    const int n = __popc(ball);
-    if (in) {
-      const int k = __popc(ball & ((1u << lane) - 1u));
-      store_pairs(st, &S[0][k], 32);
-      const float *gp = a.grad + (size_t)g * Q;
-      float gv[2 * QP];
-      gv[2 * QP - 1] = 0.f;
-      if (Q % 2 == 0 && a.grad_pairs) {  // 8-byte aligned rows: one 8-byte load per two floats
-#pragma unroll
-        for (int q = 0; q < Q; q += 2) {
-          const float2 v2 = __ldg(reinterpret_cast<const float2 *>(gp + q));
-          gv[q] = v2.x;
-          gv[q + 1] = v2.y;
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) gv[q] = __ldg(gp + q);
-      }
-#pragma unroll
-      for (int v = 0; v < QP; ++v) S[4 + v][k] = make_float4(gv[2 * v], gv[2 * v], gv[2 * v + 1], gv[2 * v + 1]);
-    }
-    __syncwarp();
+  // composites the n splats in shared memory
+  auto composite = [&](int n) {
     for (int k = 0; k < n; ++k) {
       f32x2 X, Y;
       float t0, t1;
@@ -127,7 +101,84 @@ __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
       T0 = T0 < tmin ? 0.f : T0;
       T1 = T1 < tmin ? 0.f : T1;
     }
-    __syncwarp();
+  };
+  // attribute of Gaussian g
+  auto attribute = [&](uint32_t g, float (&gv)[2 * QP]) {
+    const float *gp = a.grad + (size_t)g * Q;
+    gv[2 * QP - 1] = 0.f;
+    if (Q % 2 == 0 && a.grad_pairs) {  // 8-byte aligned rows: one 8-byte load per two floats
+#pragma unroll
+      for (int q = 0; q < Q; q += 2) {
+        const float2 v2 = __ldg(reinterpret_cast<const float2 *>(gp + q));
+        gv[q] = v2.x;
+        gv[q + 1] = v2.y;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) gv[q] = __ldg(gp + q);
+    }
+  };
+  auto store = [&](const StagedSplat &st, const float (&gv)[2 * QP], int k) {
+    store_pairs(st, &S[0][k], 32);
+#pragma unroll
+    for (int v = 0; v < QP; ++v) S[4 + v][k] = make_float4(gv[2 * v], gv[2 * v], gv[2 * v + 1], gv[2 * v + 1]);
+  };
+
+  if (kAhead) {
+    // Three batches in flight: a batch's attributes are loaded while the one before it is
+    // composited, its splats a batch earlier, their indices another batch earlier.
+    uint32_t g1 = 0, g2 = 0;
+    float4 sm1 = make_float4(0.f, 0.f, 0.f, 0.f), kc1 = sm1;
+    if (rg.x + lane < rg.y) {
+      g1 = a.pval[rg.x + lane];
+      sm1 = a.smean[g1];
+      kc1 = a.sconic[g1];
+    }
+    if (rg.x + 32 + lane < rg.y) g2 = a.pval[rg.x + 32 + lane];
+    int n0 = 0;  // splats of the previous batch
+    for (unsigned s = rg.x; s < rg.y; s += 32) {
+      if (!__any_sync(0xffffffffu, T0 + T1 > 0.f)) break;
+      const StagedSplat st = stage_splat(sm1, kc1, x0f, y0f);
+      const bool in = s + lane < rg.y && reaches_block<8>(st, kc1, amin, by, bx);
+      const unsigned ball = __ballot_sync(0xffffffffu, in);
+      float gv[2 * QP] = {};
+      if (in) attribute(g1, gv);
+      g1 = g2;
+      if (s + 32 + lane < rg.y) {
+        sm1 = a.smean[g1];
+        kc1 = a.sconic[g1];
+      }
+      if (s + 64 + lane < rg.y) g2 = a.pval[s + 64 + lane];
+      composite(n0);
+      __syncwarp();
+      if (in) store(st, gv, __popc(ball & ((1u << lane) - 1u)));
+      __syncwarp();
+      n0 = __popc(ball);
+    }
+    composite(n0);  // (stopped pixels have T = 0: no weight)
+  } else {
+    for (unsigned s = rg.x; s < rg.y; s += 32) {
+      if (!__any_sync(0xffffffffu, T0 + T1 > 0.f)) break;
+      const unsigned j = s + lane;
+      StagedSplat st;
+      uint32_t g = 0;
+      bool in = false;
+      if (j < rg.y) {
+        g = a.pval[j];
+        const float4 kc = a.sconic[g];
+        st = stage_splat(a.smean[g], kc, x0f, y0f);
+        in = reaches_block<8>(st, kc, amin, by, bx);
+      }
+      const unsigned ball = __ballot_sync(0xffffffffu, in);
+      if (in) {
+        float gv[2 * QP];
+        attribute(g, gv);
+        store(st, gv, __popc(ball & ((1u << lane) - 1u)));
+      }
+      __syncwarp();
+      composite(__popc(ball));
+      __syncwarp();
+    }
   }
   const size_t plane = (size_t)a.H * a.W;
   const size_t o = (size_t)py * a.W + px;
@@ -140,6 +191,12 @@ __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
   }
 }
 
+template <int Q>
+void launch_tiles(const RasterArgs &a, cudaStream_t st) {
+  if (a.T <= kAheadTiles) launch_k(raster_kernel<Q, true>, a.T, kRasterThreads, 0, st, a);
+  else launch_k(raster_kernel<Q, false>, a.T, kRasterThreads, 0, st, a);
+}
+
 }  // namespace
 
 cudaError_t launch_raster(const RasterArgs &a_in, cudaStream_t st) {
@@ -148,12 +205,12 @@ cudaError_t launch_raster(const RasterArgs &a_in, cudaStream_t st) {
   a.grad_pairs = (a.Q % 2 == 0 && (reinterpret_cast<uintptr_t>(a.grad) & 7u) == 0) ? 1 : 0;
   LaunchScope ls_("raster", st);
   switch (a.Q) {
-    case 1: launch_k(raster_kernel<1>, a.T, kRasterThreads, 0, st, a); break;
-    case 2: launch_k(raster_kernel<2>, a.T, kRasterThreads, 0, st, a); break;
-    case 3: launch_k(raster_kernel<3>, a.T, kRasterThreads, 0, st, a); break;
-    case 4: launch_k(raster_kernel<4>, a.T, kRasterThreads, 0, st, a); break;
-    case 6: launch_k(raster_kernel<6>, a.T, kRasterThreads, 0, st, a); break;
-    case 8: launch_k(raster_kernel<8>, a.T, kRasterThreads, 0, st, a); break;
+    case 1: launch_tiles<1>(a, st); break;
+    case 2: launch_tiles<2>(a, st); break;
+    case 3: launch_tiles<3>(a, st); break;
+    case 4: launch_tiles<4>(a, st); break;
+    case 6: launch_tiles<6>(a, st); break;
+    case 8: launch_tiles<8>(a, st); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -66,6 +66,13 @@ def test_maps_of_needles_match_oracle(hw, channels, laplacian):
     assert np.abs(gm - om)[..., ok].max() <= tol
 
 
+@pytest.mark.parametrize("hw", [(608, 1024), (609, 1024)])
+@pytest.mark.parametrize("channels,laplacian", [(1, False), (3, False), (3, True)])
+def test_maps_on_both_sides_of_the_load_ahead_line(hw, channels, laplacian):
+    """2432 tiles, the most that load ahead, and one row of tiles more; lists of 0 to 300."""
+    test_maps_of_needles_match_oracle(hw, channels, laplacian)
+
+
 @pytest.mark.parametrize("hw", [(7, 13), (24, 40), (45, 33)])
 @pytest.mark.parametrize("channels,laplacian", [(1, False), (3, False), (4, False), (1, True), (3, True)])
 def test_gradients_of_needles_match_oracle(hw, channels, laplacian):
