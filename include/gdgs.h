@@ -129,11 +129,15 @@ typedef struct gdgs_raster_opts {
   int32_t pairs_per_gaussian;
 } gdgs_raster_opts;
 
-/* Multigrid options (Sec. 2.1 lists multigrid among the linear-complexity
- * solvers; the paper fixes no parameters).
+/* Solver options (Sec. 2.1; the paper fixes no parameters).
+ * With the default omega and coarse_max_dim and both sides in 2..4096 the system
+ * is solved directly by cosine transforms in FP32, refined twice (a third time
+ * when rtol is not met); nu1, nu2 and storage then change nothing, and max_cycles
+ * bounds the refinement cycles. Any other omega or coarse_max_dim, and other
+ * sizes, take multigrid cycles. Both stop at the same residual.
  *   nu1, nu2        red-black Gauss-Seidel sweeps before / after the coarse
  *                   correction, each in 1..3                         (2, 1)
- *   max_cycles      upper bound on V-cycles, 1..64                   (30)
+ *   max_cycles      upper bound on cycles, 1..64                     (30)
  *   rtol            stop when ||rho - L u||_2 <= rtol ||rho||_2       (1e-6)
  *   coarse_max_dim  coarsen until both grid sides are <= this; the
  *                   coarsest grid is solved directly in FP64, 2..16   (8)

@@ -1,7 +1,7 @@
 // Direct Neumann solve (Eq. p2d) by cosine transforms, refined to the caller's rtol.
 // Measured on a GB300 against the multigrid cycles it takes over from: 1920x1080x3 from
-// maps 743 -> 221 us, 1355x757x3 (Bluestein) 779 -> 350 us, 3840x2160x1 1486 -> 301 us,
-// 128x96x1 220 -> 59 us; relative error of the image 1.7e-6 -> 7e-8 (1080p).
+// maps 739 -> 210 us, 1355x757x3 (Bluestein) 783 -> 293 us, 3840x2160x1 1473 -> 275 us,
+// 128x96x1 218 -> 59 us; relative error of the image 1.5e-6 -> 1e-7 (1080p).
 //
 // On the pixel grid the 5-point Neumann Laplacian is diagonal in the DCT-II modes of
 // the two sides (Sec. 2.1 lists Fourier-type solvers beside multigrid): with
@@ -205,7 +205,7 @@ cudaError_t opt_in(const FctKernels &k) {
 // The direct solve takes every number of sweeps with the default relaxation and coarsest
 // grid: a caller who sets one of these two gets the multigrid cycles he describes (all of
 // them change the way to the solution, not the solution; with 1 + 1 sweeps the multigrid
-// took 1084 us for 1617x768x4, the direct solve DIRECT us). Sides up to the longest FFT length, 4096
+// took 1084 us for 1617x768x4, the direct solve 337 us). Sides up to the longest FFT length, 4096
 // points (Bluestein's convolution of 8192 points included).
 bool fct_plan(const PoissonArgs &a, FctPlan *f) {
   if (a.omega != 1.2f || a.coarse_max_dim != 8 || !fct_enabled()) return false;

@@ -19,9 +19,9 @@
 // zero-mean solution of L u = f), built once per grid shape by Gauss-Jordan on
 // the device and cached in the workspace under a tag.
 //
-// With the default cycle options and sides up to 4096 pixels the divergence is followed
-// by the direct solve of fct.cu; the cycles below serve the other sizes and a caller's own
-// sweeps, relaxation or coarsest grid.
+// With the default relaxation and coarsest grid and sides up to 4096 pixels the divergence is
+// followed by the direct solve of fct.cu; the cycles below serve the other sizes and a
+// caller's own relaxation or coarsest grid.
 //
 // Iteration. The finest iterate u is a float-float pair (hi + lo): an FP32
 // image carries a representation error that alone gives a relative residual
@@ -2272,7 +2272,7 @@ __global__ void __launch_bounds__(256) divergence_kernel(DivArgs a, Ctrl *ctrl) 
   bool bad = false;
   float n2 = 0.f, s1 = 0.f;
   // a warp takes 128 pixels of one row, a lane every 32nd of them: one division for four
-  // pixels (a 64-bit division per pixel made this 60 us at 1617x768x4, see kDivSpan)
+  // pixels (with a 64-bit division per pixel 77 us at 1617x768x4, now 50)
   const int spans = (a.W + kDivSpan - 1) / kDivSpan, units = a.H * spans, lane = threadIdx.x & 31;
   for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < units; u += (gridDim.x * blockDim.x) >> 5) {
     const int i = u / spans, j0 = (u - i * spans) * kDivSpan + lane;
