@@ -133,8 +133,8 @@ typedef struct gdgs_raster_opts {
  * With the default omega and coarse_max_dim and both sides in 2..4096 the system
  * is solved directly by cosine transforms in FP32, refined twice (a third time
  * when rtol is not met); nu1, nu2 and storage then change nothing, and max_cycles
- * bounds the refinement cycles. Any other omega or coarse_max_dim, and other
- * sizes, take multigrid cycles. Both stop at the same residual.
+ * bounds the refinement cycles. Any other omega or coarse_max_dim, other sizes
+ * and large images whose sides have large prime factors take multigrid cycles. Both stop at the same residual.
  *   nu1, nu2        red-black Gauss-Seidel sweeps before / after the coarse
  *                   correction, each in 1..3                         (2, 1)
  *   max_cycles      upper bound on cycles, 1..64                     (30)

@@ -213,6 +213,14 @@ bool fct_plan(const PoissonArgs &a, FctPlan *f) {
   f->ex = plan_side(a.W, &f->x);
   f->ey = plan_side(a.H, &f->y);
   if (!f->ex || !f->ey) return false;
+  // Bluestein transforms cost two to three times a direct length, 0.10 ns a pixel and channel
+  // with both sides, 0.067 with one; the multigrid, whose finest passes stream at even widths,
+  // about 400 us + 0.05 ns. Large images of such sides keep it: 2176x2061x3 1423 (direct) and
+  // 1125 us, x1 520 and 728; 3840x2153x3 1656 and 1614, 2560x2153x3 1167 and 1247; at odd
+  // widths the direct solve is faster throughout (3833x2153x3 2442 and 3108).
+  const int chirps = f->x.bluestein + f->y.bluestein;
+  const long long work = (long long)a.H * a.W * a.C;
+  if (a.W % 2 == 0 && ((chirps == 2 && work > 8000000) || (chirps == 1 && work > 22000000))) return false;
   f->cycles = std::min(a.max_cycles, kFctMaxCycles);
   f->wp = (a.W + 7) & ~7;
   // the arrays of the multigrid corrections and residuals, which this path does not use

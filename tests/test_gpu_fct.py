@@ -82,6 +82,23 @@ def test_sides_outside_the_transforms_keep_the_multigrid(hw):
     assert "fct_columns" not in _profiled(maps, [0.5])
 
 
+@pytest.mark.parametrize("hwc,direct", [((2061, 2176, 1), True), ((2061, 2176, 3), False), ((2061, 2175, 3), True),
+                                        ((2153, 2560, 3), True), ((2153, 3840, 3), False), ((2160, 3840, 3), True)])
+def test_large_sides_without_a_length_of_their_own(hwc, direct):
+    """Even widths: both sides by Bluestein above 8M values, one of them above 22M, stay with
+    the multigrid; either way the solve meets rtol."""
+    H, W, C = hwc
+    rho = torch.randn((C, H, W), device="cuda", generator=torch.Generator("cuda").manual_seed(H + W))
+    rho -= rho.mean(dim=(1, 2), keepdim=True)
+    img = torch.empty_like(rho)
+    ws = torch.empty(G.workspace_size(0, C, W, H, None, None), dtype=torch.uint8, device="cuda")
+    G.profile_begin()
+    G.poisson_reconstruct_rho(rho, [0.5] * C, img, ws)
+    names = G.profile_end()
+    st = G.sync_status(ws)
+    assert st["status"] == 0 and ("fct_columns" in names) == direct, (st, list(names))
+
+
 @pytest.mark.parametrize("storage", [0, 1, 2])
 @pytest.mark.parametrize("hw", [(150, 210), (101, 67)])
 def test_direct_and_multigrid_agree_over_the_options(hw, storage):
