@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kHistThreads) depth_hist_kernel(DepthSort a, S
 // blocks an SM (64 registers without spills) were the fastest of 1536 .. 8192; ranking by
 // votes over the digit's bits (32 instructions) came out equal, __match_any_sync 20 % slower.
 // The seven passes of a 3840x2160 view (1M Gaussians, 16.4M pairs) 333 us, of 1920x1080 (200k,
-// 2.7M) 88 us, launch gaps included; block histogram, scan and scatter kernels for each pass
+// 1.3M) 88 us, launch gaps included; block histogram, scan and scatter kernels for each pass
 // and a pass for the tile ranges took 735 and 196 us.
 // kKind: kSortPlain; kSortLow: ranked by the secondary keys, values are the indices and the
 // keys written are the primary ones; kSortRanges: the last pass over the pairs, whose output
