@@ -5,7 +5,7 @@
 
 #include <algorithm>
 
-#include "gdgs_internal.cuh"
+#include "fct.cuh"
 
 namespace gdgs {
 
@@ -650,7 +650,7 @@ int gdgs_sync_status(const void *ws, gdgs_solve_stats *stats, void *stream) {
     for (int i = 0; i < c.channels && i < GDGS_MAX_CHANNELS; ++i) {
       const int kf = c.kf_c[i];
       if (kf < 0 || kf > c.direct) return GDGS_ERR_CUDA;  // not a finished solve's block
-      const double a = c.rnorm2[fct_slot(0, i)], b = c.rnorm2[fct_slot(kf, i)];
+      const double a = c.rnorm2[c.rtol >= 1.0 ? fct_sq_slot(i) : fct_slot(0, i)], b = kf ? c.rnorm2[fct_slot(kf, i)] : a;
       r0 += a;
       rf += b;
       met = met && b <= thr * a;

@@ -58,28 +58,39 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
   griddep_enter();
   const int c = blockIdx.y;
   __shared__ int s_kf, s_skip;
-  __shared__ float s_shift;
+  __shared__ float s_shift, s_hi, s_lo;
   if (threadIdx.x == 0) {
     bool done;
-    const int kf = fct_cycles_done(a.ctrl, c, a.inv_cells, k - 1, &done);
+    const float hi = fct_mean_hi(a.ctrl, c, a.inv_cells), lo = a.ctrl->rho_mean[c];
+    double su[kFctMaxCycles];  // sums of the corrections
+#pragma unroll
+    for (int q = 0; q < kFctMaxCycles; ++q) su[q] = a.ctrl->sum_u[q + 1][c];
+    const int kf = fct_cycles_done(a.ctrl, c, k - 1, &done);
     s_skip = done && !first;
     s_kf = done ? kf : k;
     float mc = a.mean[0];
 #pragma unroll
     for (int i = 1; i < GDGS_MAX_CHANNELS; ++i)
       if (i == c) mc = a.mean[i];
-    double sum = 0.0;  // of u: the sums of its corrections
-    for (int q = 1; q <= s_kf; ++q) sum += a.ctrl->sum_u[q][c];
+    double sum = 0.0;  // of u
+#pragma unroll
+    for (int q = 0; q < kFctMaxCycles; ++q)
+      if (q < (done ? kf : k)) sum += su[q];
     s_shift = (float)((double)mc - sum * a.inv_cells);
+    s_hi = hi;
+    s_lo = lo;
     if (blockIdx.x == 0 && !s_skip) {
       a.ctrl->kf_c[c] = s_kf;
       a.ctrl->mean_set[c] = mc;
-      a.ctrl->rnorm2[fct_slot(0, c)] = fct_r0(a.ctrl, c, a.inv_cells);
+      if (a.rtol2 >= 1.0) {  // no pass ran that records it
+        const double m = a.ctrl->rho_sum[c];
+        a.ctrl->rnorm2[fct_sq_slot(c)] = fmax(a.ctrl->rho_sq[c] - m * m * a.inv_cells, 0.0);
+      }
     }
   }
   __syncthreads();
   if (s_skip) return;
-  const float mean_rho = fct_block_mean(a, c);
+  const float hi = s_hi, lo = s_lo;
   const int kf = s_kf, W = a.W, H = a.H;
   const float shift = s_shift;
   const size_t plane = (size_t)H * W;
@@ -107,8 +118,8 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
     row(rho, p, r);
 #pragma unroll
     for (int d = 0; d < V; ++d) l[d + 1] = 0.f;
-    // r -= L of one part of the iterate
-    auto minus_lap = [&](const float *u, float *c) {
+    // L of one part of the iterate
+    auto lap = [&](const float *u, float *c, float *out) {
       float s[V], n[V];
       row(u, p, c + 1);
       row(u, ps, s);
@@ -116,14 +127,20 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
       c[0] = j0 > 0 ? __ldg(u + p - 1) : c[1];
       c[V + 1] = j0 + V < W ? __ldg(u + p + V) : c[V];
 #pragma unroll
-      for (int d = 0; d < V; ++d) r[d] -= fct_lap(c[d + 1], c[d + 2], c[d], s[d], n[d]);
+      for (int d = 0; d < V; ++d) out[d] = fct_lap(c[d + 1], c[d + 2], c[d], s[d], n[d]);
     };
-    minus_lap(uh, h);
-    if (kf > 1) minus_lap(ul, l);
+    float lu[V];
+    lap(uh, h, lu);
+#pragma unroll
+    for (int d = 0; d < V; ++d) r[d] = fct_residual(r[d], hi, lo, lu[d]);
+    if (kf > 1) {
+      lap(ul, l, lu);
+#pragma unroll
+      for (int d = 0; d < V; ++d) r[d] -= lu[d];
+    }
     float o[V];
 #pragma unroll
     for (int d = 0; d < V; ++d) {
-      r[d] -= mean_rho;
       r2 = fmaf(r[d], r[d], r2);
       o[d] = h[d + 1] + (l[d + 1] + shift);
     }
@@ -260,7 +277,9 @@ cudaError_t run_fct(const PoissonArgs &a, const FctPlan &f, const float *rho, fl
   fa.ulo = ulo;
   fa.spec = f.spec;
   fa.image = a.image;
-  fa.inv_cells = 1.0 / ((double)a.H * a.W);
+  fa.cells = (double)a.H * a.W;
+  fa.inv_cells = 1.0 / fa.cells;
+  fa.rtol2 = (double)a.rtol * a.rtol;
   for (int c = 0; c < GDGS_MAX_CHANNELS; ++c) fa.mean[c] = a.mean[c];
   fa.ctrl = a.ctrl;
   cudaError_t e = opt_in(*f.ex);

@@ -27,7 +27,7 @@ struct FctArgs {
   int C, H, W, wp;
   const float *rho;
   float *uhi, *ulo, *spec, *image;
-  double inv_cells;
+  double cells, inv_cells, rtol2;
   float mean[GDGS_MAX_CHANNELS];
   Ctrl *ctrl;
 };
@@ -95,38 +95,79 @@ __device__ __forceinline__ void fct_build_tables(const FctSide &d, int tid, int 
   }
 }
 
-// ||rho - mean||^2 of channel c, and whether it needs no further cycle after `k` cycles
+// The mean of rho in two parts: `hi`, the float nearest to the sum the divergence left (its
+// FP32 partial sums are off by ~1e-8 of a mean that dominates the field), is known from the
+// start and what the transforms work on is rho - hi; `lo`, the mean of that, is its lowest
+// cosine coefficient, which the first column pass leaves in ctrl->rho_mean.
+__device__ __forceinline__ float fct_mean_hi(const Ctrl *ctrl, int c, double inv_cells) {
+  return (float)(ctrl->rho_sum[c] * inv_cells);
+}
+// Where the first rows pass leaves sum (rho - hi)^2 (for rtol >= 1, where no pass but the finalize
+// runs, that leaves ||rho - mean||^2), and the first rows-back pass the square of the residual
+// that rtol asks for.
+__host__ __device__ constexpr int fct_sq_slot(int c) { return fct_slot(kFctMaxCycles + 2, c); }
+__host__ __device__ constexpr int fct_goal_slot(int c) { return fct_slot(kFctMaxCycles + 3, c); }
+
+// By one thread of the first rows-back pass, which has the low part and `sq`: ||rho - mean||^2 (0
+// where the difference is only the rounding of its two terms: a constant field) and the goal, so
+// that the blocks of the later passes compare and do not compute in FP64 (0.7 us a launch).
+__device__ __forceinline__ void fct_record_goal(const FctArgs &a, int c, float lo, double sq) {
+  const double m2 = (double)lo * lo * a.cells, r0 = sq - m2, r = r0 > 1e-5 * m2 ? r0 : 0.0;
+  a.ctrl->rnorm2[fct_slot(0, c)] = r;
+  a.ctrl->rnorm2[fct_goal_slot(c)] = a.rtol2 * r;
+}
+
+// Whether channel c needs no further cycle after `k` cycles, and the number it has had
 // (its residual after 1 .. k cycles is recorded, 0 cycles: a zero right-hand side). The
 // rounding of the forward transforms is white noise of ~1e-7 of rho, which the division by
 // lambda amplifies in the lowest modes (5e-5 of the image on 200 x 3 pixels at a relative
 // residual of 4e-7), so the first cycle ends a solve only far below rtol.
-__device__ __forceinline__ double fct_r0(const Ctrl *ctrl, int c, double inv_cells) {
-  const double s = ctrl->rho_sum[c];
-  return fmax(ctrl->rho_sq[c] - s * s * inv_cells, 0.0);
-}
-__device__ __forceinline__ int fct_cycles_done(const Ctrl *ctrl, int c, double inv_cells, int k, bool *done) {
-  const double thr = ctrl->rtol * ctrl->rtol * fct_r0(ctrl, c, inv_cells);
-  if (ctrl->rtol * ctrl->rtol >= 1.0 || fct_r0(ctrl, c, inv_cells) == 0.0) {
-    *done = true;
-    return 0;
-  }
-  for (int q = 1; q <= k; ++q)
-    if (ctrl->rnorm2[fct_slot(q, c)] <= (q == 1 ? 1e-4 * thr : thr)) {
-      *done = true;
-      return q;
-    }
+__device__ __forceinline__ int fct_cycles_done(const Ctrl *ctrl, int c, int k, bool *done) {
+  // all loads at once (each takes most of a microsecond, and every block waits for them)
+  const double r0 = ctrl->rnorm2[fct_slot(0, c)], goal = ctrl->rnorm2[fct_goal_slot(c)];
+  double r[kFctMaxCycles];
+#pragma unroll
+  for (int q = 1; q <= kFctMaxCycles; ++q) r[q - 1] = ctrl->rnorm2[fct_slot(q, c)];
+  int n = k;
   *done = false;
-  return k;
+#pragma unroll
+  for (int q = kFctMaxCycles; q >= 1; --q)
+    if (q <= k && r[q - 1] <= (q == 1 ? 1e-4 * goal : goal)) {
+      *done = true;
+      n = q;
+    }
+  if (r0 == 0.0) {
+    *done = true;
+    n = 0;
+  }
+  return n;
 }
-__device__ __forceinline__ bool fct_block_done(const FctArgs &a, int c, int k) {
-  __shared__ int s_done;
+// The mean of channel c's rho, and whether a pass has nothing to do there (skip): after `k`
+// cycles, as above. k < 0: a pass of the first cycle, before the goal is known, which only a zero
+// field (kFctRows) or one that is its mean (kFctFirst) can skip, or any for rtol >= 1.
+enum { kFctRows = -2, kFctFirst = -1 };
+struct FctChannel {
+  float hi, lo;
+  bool skip;
+  double sq;  // (k < 0)
+};
+__device__ __forceinline__ FctChannel fct_block_channel(const FctArgs &a, int c, int k) {
+  __shared__ FctChannel s_c;
   if (threadIdx.x == 0) {
-    bool d;
-    fct_cycles_done(a.ctrl, c, a.inv_cells, k, &d);
-    s_done = d;
+    FctChannel f;
+    f.hi = fct_mean_hi(a.ctrl, c, a.inv_cells);
+    f.lo = a.ctrl->rho_mean[c];
+    f.sq = 0.0;
+    if (k < 0) {
+      f.sq = *(k == kFctRows ? &a.ctrl->rho_sq[c] : &a.ctrl->rnorm2[fct_sq_slot(c)]);
+      f.skip = (a.rtol2 >= 1.0) | (f.sq == 0.0);
+    } else {
+      fct_cycles_done(a.ctrl, c, k, &f.skip);
+    }
+    s_c = f;
   }
   __syncthreads();
-  return s_done != 0;
+  return s_c;
 }
 
 // Block-wide sum; the result is valid in thread 0.
@@ -143,11 +184,11 @@ __device__ __forceinline__ float fct_block_sum(float v) {
   return s;
 }
 
-// The residual rho - mean - L u without rounding errors that matter, in plain FP32: the
+// L u without rounding errors that matter, in plain FP32: the
 // first correction u_1 is stored rounded to multiples of one power of two g per channel,
 // about ulp(8 rms(u_1)) (fct_grid), so its differences and their sums are exact (below
-// 2^24 g; beyond, they round relative to themselves), and rho minus that sum loses nothing
-// where the two cancel. u can be 1e5 times as large as L u (smooth right-hand sides,
+// 2^24 g; beyond, they round relative to themselves), and rho - mean minus that sum loses nothing
+// where the two cancel (fct_residual). u can be 1e5 times as large as L u (smooth right-hand sides,
 // images spanning hundreds); with u_1 rounded to each value's own ulp the same sums were
 // off by more than the 1e-6 of rho that a cycle has to see, and error-free transformations
 // cost 70 instructions a pixel. The rounding itself is ~1e-6 of rms(u_1), like that of the
@@ -165,12 +206,15 @@ __device__ __forceinline__ float fct_grid(double sum2) {
 }
 __host__ __device__ constexpr int fct_grid_slot(int c) { return fct_slot(kFctMaxCycles + 1, c); }
 
-// The mean of rho over channel c.
-__device__ __forceinline__ float fct_block_mean(const FctArgs &a, int c) {
-  __shared__ float s_m;
-  if (threadIdx.x == 0) s_m = (float)(a.ctrl->rho_sum[c] * a.inv_cells);
-  __syncthreads();
-  return s_m;
+// What is left of rho - mean when the exact sums `lap` of the parts of the iterate that cancel it
+// go first. The mean comes off first (next to a mean of 30 deviations, rho - lap would keep 5 bits fewer
+// of the residual: images 1e-4 to 3e-2 of their range off, with a residual of exactly 0), with
+// the rounding error of that difference kept (Knuth's two-sum), or rho would be solved for
+// to 2^-24 only.
+__device__ __forceinline__ float fct_residual(float rho, float hi, float lo, float lap) {
+  const float t = __fsub_rn(rho, hi), b = __fsub_rn(t, rho);
+  const float err = __fsub_rn(__fsub_rn(rho, __fsub_rn(t, b)), __fadd_rn(hi, b));
+  return __fadd_rn(__fsub_rn(t, lap), __fsub_rn(err, lo));
 }
 
 }  // namespace gdgs

@@ -468,8 +468,8 @@ __device__ __forceinline__ void dft(float2 *S, const FctSide &d, int t, bool sme
 // back of a solve: 56 registers 652 us, 64 670 us, 80 704 us, 48 655 us (and slower at 1080p).
 constexpr int blocks_per_sm(int threads) { return cmax(1, 65536 / (56 * ceil_div(threads, 32) * 32)); }
 
-// Rows forward (kc: cycle; cycle 0 transforms rho, later ones the residual of the
-// iterate, whose norm cycle 1 records).
+// Rows forward (kc: cycle; cycle 0 transforms rho less the high part of its mean, later ones the
+// residual of the iterate; cycles 0 and 1 record the norm of what they transform).
 template <class F, bool BL>
 __global__ void __launch_bounds__(ceil_div(F::G_ROWS * F::TP, 32) * 32, blocks_per_sm(F::G_ROWS * F::TP))
 fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
@@ -479,7 +479,8 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
   const int c = blockIdx.y;
   // the residual after one cycle is recorded by this launch itself (kc == 1), after two by
   // the finalize pass before it
-  if (fct_block_done(a, c, kc == 1 ? 0 : kc)) return;
+  const FctChannel ch = fct_block_channel(a, c, kc == 0 ? kFctRows : kc == 1 ? 0 : kc);
+  if (ch.skip) return;
   const int g = threadIdx.x / TP, t = g < G ? (int)threadIdx.x - g * TP : TP;
   float2 *S = fct_sm + (g < G ? g : 0) * F::template Layout<1>::SLOTS;
   const int W = a.W, H = a.H;
@@ -489,15 +490,12 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
   const float *rho = a.rho + c * plane;
   float acc = 0.f;
   if (kc > 0) {
-    const float mean_rho = fct_block_mean(a, c);
     const float *uh = a.uhi + c * plane, *ul = a.ulo + c * plane;
-    // residual of columns j, j + 1 of both rows: the field given minus L of the part u
-    auto minus_lap = [&](const float *u, int j, float2 &ra, float2 &rb) {
+    // L u of the part u at columns j, j + 1 of both rows
+    auto lap = [&](const float *u, int j, float2 &la, float2 &lb) {
       const Patch h = ld_patch(u, ia, j, W, H);
-      ra.x -= fct_lap(h.a.x, h.a.y, h.al, h.b.x, h.n.x);
-      ra.y -= fct_lap(h.a.y, h.ar, h.a.x, h.b.y, h.n.y);
-      rb.x -= fct_lap(h.b.x, h.b.y, h.bl, h.s.x, h.a.x);
-      rb.y -= fct_lap(h.b.y, h.br, h.b.x, h.s.y, h.a.y);
+      la = make_float2(fct_lap(h.a.x, h.a.y, h.al, h.b.x, h.n.x), fct_lap(h.a.y, h.ar, h.a.x, h.b.y, h.n.y));
+      lb = make_float2(fct_lap(h.b.x, h.b.y, h.bl, h.s.x, h.a.x), fct_lap(h.b.y, h.br, h.b.x, h.s.y, h.a.y));
     };
     if (t < TP) {
 #pragma unroll 2
@@ -505,12 +503,18 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
         const int j = 2 * m;
         float2 ra = make_float2(0.f, 0.f), rb = ra;
         if (va) {
+          float2 la, lb;
           ra = ld_pair(rho + (size_t)ia * W, j, W);
           if (vb) rb = ld_pair(rho + (size_t)(ia + 1) * W, j, W);
-          minus_lap(uh, j, ra, rb);
-          if (kc > 1) minus_lap(ul, j, ra, rb);
-          ra = make_float2(ra.x - mean_rho, ra.y - mean_rho);
-          rb = vb ? make_float2(rb.x - mean_rho, rb.y - mean_rho) : make_float2(0.f, 0.f);
+          lap(uh, j, la, lb);
+          ra = make_float2(fct_residual(ra.x, ch.hi, ch.lo, la.x), fct_residual(ra.y, ch.hi, ch.lo, la.y));
+          rb = make_float2(fct_residual(rb.x, ch.hi, ch.lo, lb.x), fct_residual(rb.y, ch.hi, ch.lo, lb.y));
+          if (kc > 1) {
+            lap(ul, j, la, lb);
+            ra = make_float2(ra.x - la.x, ra.y - la.y);
+            rb = make_float2(rb.x - lb.x, rb.y - lb.y);
+          }
+          if (!vb) rb = make_float2(0.f, 0.f);
           acc = fmaf(ra.x, ra.x, acc);
           acc = fmaf(rb.x, rb.x, acc);
           if (j + 1 < W) {
@@ -534,7 +538,9 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
       gather<M>(v, j0, [&](int i) -> float2 {
         if (BL && i >= W) return make_float2(0.f, 0.f);
         const int j = 2 * i < W ? 2 * i : 2 * (W - 1 - i) + 1;
-        return make_float2(va ? __ldg(ra + j) : 0.f, vb ? __ldg(ra + W + j) : 0.f);
+        const float2 r = make_float2(va ? __ldg(ra + j) - ch.hi : 0.f, vb ? __ldg(ra + W + j) - ch.hi : 0.f);
+        acc = fmaf(r.x, r.x, fmaf(r.y, r.y, acc));
+        return r;
       });
     }
   });
@@ -557,9 +563,9 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
       }
     }
   }
-  if (kc == 1) {
+  if (kc <= 1) {
     acc = fct_block_sum(acc);
-    if (threadIdx.x == 0) atomicAdd(&a.ctrl->rnorm2[fct_slot(1, c)], (double)acc);
+    if (threadIdx.x == 0) atomicAdd(&a.ctrl->rnorm2[kc == 0 ? fct_sq_slot(c) : fct_slot(1, c)], (double)acc);
   }
 }
 
@@ -571,7 +577,7 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
   extern __shared__ float2 fct_sm[];
   constexpr int TP = F::TP, G = F::G_COLS;
   const int c = blockIdx.y;
-  if (fct_block_done(a, c, kc)) return;
+  if (fct_block_channel(a, c, kc == 0 ? kFctFirst : kc).skip) return;
   const int g = threadIdx.x % G;
   const int t = min((int)threadIdx.x / G, TP);
   float2 *S = fct_sm + g;
@@ -613,6 +619,7 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
         }
         Quad q = dct_post(z, zn, tk);
         const float lk = __ldg(a.y.s2 + k), ln = __ldg(a.y.s2 + kn);
+        if (kc == 0 && k == 0 && ja == 0) a.ctrl->rho_mean[c] = -scale * q.ak;
         q.ak = (k == 0 && ja == 0) ? 0.f : q.ak * __fdividef(scale, lk + lxa);
         q.bk = q.bk * __fdividef(scale, lk + lxb);
         q.an = k == 0 ? 0.f : q.an * __fdividef(scale, ln + lxa);
@@ -662,7 +669,9 @@ fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
   extern __shared__ float2 fct_sm[];
   constexpr int TP = F::TP, G = F::G_ROWS;
   const int c = blockIdx.y;
-  if (fct_block_done(a, c, kc)) return;
+  const FctChannel ch = fct_block_channel(a, c, kc == 0 ? kFctFirst : kc);
+  if (ch.skip) return;
+  if (kc == 0 && blockIdx.x == 0 && threadIdx.x == 0) fct_record_goal(a, c, ch.lo, ch.sq);
   const int g = threadIdx.x / TP, t = g < G ? (int)threadIdx.x - g * TP : TP;
   float2 *S = fct_sm + (g < G ? g : 0) * F::template Layout<1>::SLOTS;
   const int W = a.W, H = a.H;
