@@ -12,8 +12,8 @@
 //   rows back inverse DCT along x: the correction e
 // FP32 rounding of e leaves a relative residual of ~1e-5 (it is the size of the image's
 // own FP32 representation error), and the next cycle solves for exactly that: the
-// residual is evaluated without rounding errors that matter (fct_lap), so two cycles
-// reach ~1e-7 or less. The multigrid needs 4-6 cycles, each a chain of ~12 dependent
+// residual is evaluated without rounding errors that matter (fct_lap, FctResidual), so two
+// cycles reach ~1e-7 or less, three 1e-9 (3e-8 where the field is the lowest mode of 3800 points). The multigrid needs 4-6 cycles, each a chain of ~12 dependent
 // launches whose small levels leave the GPU idle (1080p, three channels: 150 us per
 // cycle, all latency); here every launch covers all channels and every SM.
 //
@@ -53,7 +53,8 @@ namespace {
 
 // After `k` cycles: image = u + (m_c - mean u) of the iterate channel c stopped at, and
 // (when that is the k-th) its residual. Skipped when an earlier call already finished c.
-template <int V>
+// Third: the iterate has a third part (k = 3).
+template <int V, bool Third>
 __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant__ FctArgs a, int k, int first) {
   griddep_enter();
   const int c = blockIdx.y;
@@ -105,7 +106,6 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
       for (int d = 0; d < V; ++d) img[p + d] = 0.f + (0.f + shift);
       continue;
     }
-    const int ps = i + 1 < H ? p + W : p, pn = i > 0 ? p - W : p;
     auto row = [&](const float *src, int o, float *dst) {
       if constexpr (V == 4) {
         const float4 v = __ldg(reinterpret_cast<const float4 *>(src + o));
@@ -119,28 +119,44 @@ __global__ void __launch_bounds__(256) fct_finalize_kernel(const __grid_constant
 #pragma unroll
     for (int d = 0; d < V; ++d) l[d + 1] = 0.f;
     // L of one part of the iterate
-    auto lap = [&](const float *u, float *c, float *out) {
+    auto lap = [&](const float *u, int pitch, float *c, float *out) {
       float s[V], n[V];
-      row(u, p, c + 1);
-      row(u, ps, s);
-      row(u, pn, n);
-      c[0] = j0 > 0 ? __ldg(u + p - 1) : c[1];
-      c[V + 1] = j0 + V < W ? __ldg(u + p + V) : c[V];
+      const int o = i * pitch + j0;
+      row(u, o, c + 1);
+      row(u, i + 1 < H ? o + pitch : o, s);
+      row(u, i > 0 ? o - pitch : o, n);
+      c[0] = j0 > 0 ? __ldg(u + o - 1) : c[1];
+      c[V + 1] = j0 + V < W ? __ldg(u + o + V) : c[V];
 #pragma unroll
       for (int d = 0; d < V; ++d) out[d] = fct_lap(c[d + 1], c[d + 2], c[d], s[d], n[d]);
     };
-    float lu[V];
-    lap(uh, h, lu);
+    float lu[V], rl[V];
+    lap(uh, W, h, lu);
 #pragma unroll
-    for (int d = 0; d < V; ++d) r[d] = fct_residual(r[d], hi, lo, lu[d]);
+    for (int d = 0; d < V; ++d) {
+      FctResidual x(r[d], hi, lo);
+      x.minus(lu[d]);
+      r[d] = x.hi;
+      rl[d] = x.lo;
+    }
     if (kf > 1) {
-      lap(ul, l, lu);
+      lap(ul, W, l, lu);
 #pragma unroll
-      for (int d = 0; d < V; ++d) r[d] -= lu[d];
+      for (int d = 0; d < V; ++d) r[d] -= lu[d];  // (what is left is about as large: nothing is lost)
+    }
+    if (Third && kf > 2) {
+      float t[V + 2];
+      lap(a.spec + (size_t)c * H * a.wp, a.wp, t, lu);
+#pragma unroll
+      for (int d = 0; d < V; ++d) {
+        rl[d] -= lu[d];
+        l[d + 1] += t[d + 1];
+      }
     }
     float o[V];
 #pragma unroll
     for (int d = 0; d < V; ++d) {
+      r[d] += rl[d];
       r2 = fmaf(r[d], r[d], r2);
       o[d] = h[d + 1] + (l[d + 1] + shift);
     }
@@ -275,6 +291,7 @@ cudaError_t run_fct(const PoissonArgs &a, const FctPlan &f, const float *rho, fl
   fa.rho = rho;
   fa.uhi = uhi;
   fa.ulo = ulo;
+  fa.tight = a.rtol < 1e-6f;
   fa.spec = f.spec;
   fa.image = a.image;
   fa.cells = (double)a.H * a.W;
@@ -312,8 +329,9 @@ cudaError_t run_fct(const PoissonArgs &a, const FctPlan &f, const float *rho, fl
     if (k > 0 || f.cycles == 1) {
       const int first = k == std::min(1, f.cycles - 1);
       LaunchScope ls_("finalize", st);
-      if (V == 4) launch_k(fct_finalize_kernel<4>, fg, 256, 0, st, fa, k + 1, first);
-      else launch_k(fct_finalize_kernel<1>, fg, 256, 0, st, fa, k + 1, first);
+      const auto fin = V == 4 ? (k > 1 ? fct_finalize_kernel<4, true> : fct_finalize_kernel<4, false>)
+                              : (k > 1 ? fct_finalize_kernel<1, true> : fct_finalize_kernel<1, false>);
+      launch_k(fin, fg, 256, 0, st, fa, k + 1, first);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

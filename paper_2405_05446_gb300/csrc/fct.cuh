@@ -26,7 +26,8 @@ struct FctArgs {
   FctSide x, y;
   int C, H, W, wp;
   const float *rho;
-  float *uhi, *ulo, *spec, *image;
+  float *uhi, *ulo, *spec, *image;  // uhi, ulo: the first and second correction
+  int tight;  // the second part goes to a grid too (fct_back_kernel)
   double cells, inv_cells, rtol2;
   float mean[GDGS_MAX_CHANNELS];
   Ctrl *ctrl;
@@ -98,7 +99,8 @@ __device__ __forceinline__ void fct_build_tables(const FctSide &d, int tid, int 
 // The mean of rho in two parts: `hi`, the float nearest to the sum the divergence left (its
 // FP32 partial sums are off by ~1e-8 of a mean that dominates the field), is known from the
 // start and what the transforms work on is rho - hi; `lo`, the mean of that, is its lowest
-// cosine coefficient, which the first column pass leaves in ctrl->rho_mean.
+// cosine coefficient, which the column passes leave in ctrl->rho_mean (the later ones what the
+// rounding of the transform left of it, 1e-8 of the field's deviation).
 __device__ __forceinline__ float fct_mean_hi(const Ctrl *ctrl, int c, double inv_cells) {
   return (float)(ctrl->rho_sum[c] * inv_cells);
 }
@@ -142,10 +144,28 @@ __device__ __forceinline__ int fct_cycles_done(const Ctrl *ctrl, int c, int k, b
   }
   return n;
 }
-// The mean of channel c's rho, and whether a pass has nothing to do there (skip): after `k`
-// cycles, as above. k < 0: a pass of the first cycle, before the goal is known, which only a zero
-// field (kFctRows) or one that is its mean (kFctFirst) can skip, or any for rtol >= 1.
+// Whether a pass has nothing to do in channel c: after `k` cycles, as above. k < 0: a pass of the
+// first cycle, before the goal is known, which only a zero field (kFctRows) or one that is its
+// mean (kFctFirst) can skip, or any for rtol >= 1; *sq is then the sum of squares it went by.
 enum { kFctRows = -2, kFctFirst = -1 };
+__device__ __forceinline__ bool fct_skip(const FctArgs &a, int c, int k, double *sq) {
+  bool skip;
+  if (k < 0) {
+    *sq = *(k == kFctRows ? &a.ctrl->rho_sq[c] : &a.ctrl->rnorm2[fct_sq_slot(c)]);
+    skip = (a.rtol2 >= 1.0) | (*sq == 0.0);
+  } else {
+    fct_cycles_done(a.ctrl, c, k, &skip);
+  }
+  return skip;
+}
+__device__ __forceinline__ bool fct_block_skip(const FctArgs &a, int c, int k) {
+  __shared__ bool s_skip;
+  double sq;
+  if (threadIdx.x == 0) s_skip = fct_skip(a, c, k, &sq);
+  __syncthreads();
+  return s_skip;
+}
+// The same with the mean of the channel's rho.
 struct FctChannel {
   float hi, lo;
   bool skip;
@@ -158,12 +178,7 @@ __device__ __forceinline__ FctChannel fct_block_channel(const FctArgs &a, int c,
     f.hi = fct_mean_hi(a.ctrl, c, a.inv_cells);
     f.lo = a.ctrl->rho_mean[c];
     f.sq = 0.0;
-    if (k < 0) {
-      f.sq = *(k == kFctRows ? &a.ctrl->rho_sq[c] : &a.ctrl->rnorm2[fct_sq_slot(c)]);
-      f.skip = (a.rtol2 >= 1.0) | (f.sq == 0.0);
-    } else {
-      fct_cycles_done(a.ctrl, c, k, &f.skip);
-    }
+    f.skip = fct_skip(a, c, k, &f.sq);
     s_c = f;
   }
   __syncthreads();
@@ -188,7 +203,7 @@ __device__ __forceinline__ float fct_block_sum(float v) {
 // first correction u_1 is stored rounded to multiples of one power of two g per channel,
 // about ulp(8 rms(u_1)) (fct_grid), so its differences and their sums are exact (below
 // 2^24 g; beyond, they round relative to themselves), and rho - mean minus that sum loses nothing
-// where the two cancel (fct_residual). u can be 1e5 times as large as L u (smooth right-hand sides,
+// where the two cancel (FctResidual). u can be 1e5 times as large as L u (smooth right-hand sides,
 // images spanning hundreds); with u_1 rounded to each value's own ulp the same sums were
 // off by more than the 1e-6 of rho that a cycle has to see, and error-free transformations
 // cost 70 instructions a pixel. The rounding itself is ~1e-6 of rms(u_1), like that of the
@@ -204,17 +219,26 @@ __device__ __forceinline__ float fct_grid(double sum2) {
   if (!(rms8 > 0.f) || !(rms8 < 1e37f)) return 0.f;
   return 3.f * exp2f(ceilf(log2f(rms8)));
 }
-__host__ __device__ constexpr int fct_grid_slot(int c) { return fct_slot(kFctMaxCycles + 1, c); }
-
-// What is left of rho - mean when the exact sums `lap` of the parts of the iterate that cancel it
-// go first. The mean comes off first (next to a mean of 30 deviations, rho - lap would keep 5 bits fewer
-// of the residual: images 1e-4 to 3e-2 of their range off, with a residual of exactly 0), with
-// the rounding error of that difference kept (Knuth's two-sum), or rho would be solved for
-// to 2^-24 only.
-__device__ __forceinline__ float fct_residual(float rho, float hi, float lo, float lap) {
-  const float t = __fsub_rn(rho, hi), b = __fsub_rn(t, rho);
-  const float err = __fsub_rn(__fsub_rn(rho, __fsub_rn(t, b)), __fadd_rn(hi, b));
-  return __fadd_rn(__fsub_rn(t, lap), __fsub_rn(err, lo));
+// Where the sum of squares of the correction of cycle 0 and of cycle 1 goes.
+__host__ __device__ constexpr int fct_grid_slot(int cycle, int c) {
+  return fct_slot(kFctMaxCycles + (cycle ? 4 : 1), c);
 }
+
+// What is left of rho - mean after the exact sums L u of the iterate's parts, as an unevaluated
+// sum hi + lo whose differences keep their rounding errors (Knuth's two-sum). The mean comes
+// off first: next to a mean of 30 deviations, rho - L u would keep 5 bits fewer of the residual
+// (images 1e-4 to 3e-2 of their range off, with a residual of exactly 0). And the residual after
+// one part can exceed rho itself (smooth fields: six times at 4096 points), where rounding it to
+// FP32 would leave 1e-7 of rho for good.
+struct FctResidual {
+  float hi, lo;
+  __device__ __forceinline__ FctResidual(float rho, float mean_hi, float mean_lo) : hi(rho), lo(-mean_lo) { minus(mean_hi); }
+  __device__ __forceinline__ void minus(float x) {
+    const float t = __fsub_rn(hi, x), b = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fsub_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fadd_rn(x, b)));
+    hi = t;
+  }
+  __device__ __forceinline__ float value() const { return __fadd_rn(hi, lo); }
+};
 
 }  // namespace gdgs

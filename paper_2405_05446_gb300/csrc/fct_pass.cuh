@@ -506,14 +506,18 @@ fct_rows_kernel(const __grid_constant__ FctArgs a, int kc) {
           float2 la, lb;
           ra = ld_pair(rho + (size_t)ia * W, j, W);
           if (vb) rb = ld_pair(rho + (size_t)(ia + 1) * W, j, W);
-          lap(uh, j, la, lb);
-          ra = make_float2(fct_residual(ra.x, ch.hi, ch.lo, la.x), fct_residual(ra.y, ch.hi, ch.lo, la.y));
-          rb = make_float2(fct_residual(rb.x, ch.hi, ch.lo, lb.x), fct_residual(rb.y, ch.hi, ch.lo, lb.y));
-          if (kc > 1) {
-            lap(ul, j, la, lb);
-            ra = make_float2(ra.x - la.x, ra.y - la.y);
-            rb = make_float2(rb.x - lb.x, rb.y - lb.y);
-          }
+          FctResidual r[4] = {{ra.x, ch.hi, ch.lo}, {ra.y, ch.hi, ch.lo}, {rb.x, ch.hi, ch.lo}, {rb.y, ch.hi, ch.lo}};
+          auto minus_lap = [&](const float *u) {
+            lap(u, j, la, lb);
+            r[0].minus(la.x);
+            r[1].minus(la.y);
+            r[2].minus(lb.x);
+            r[3].minus(lb.y);
+          };
+          minus_lap(uh);
+          if (kc > 1) minus_lap(ul);
+          ra = make_float2(r[0].value(), r[1].value());
+          rb = make_float2(r[2].value(), r[3].value());
           if (!vb) rb = make_float2(0.f, 0.f);
           acc = fmaf(ra.x, ra.x, acc);
           acc = fmaf(rb.x, rb.x, acc);
@@ -577,7 +581,7 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
   extern __shared__ float2 fct_sm[];
   constexpr int TP = F::TP, G = F::G_COLS;
   const int c = blockIdx.y;
-  if (fct_block_channel(a, c, kc == 0 ? kFctFirst : kc).skip) return;
+  if (fct_block_skip(a, c, kc == 0 ? kFctFirst : kc)) return;
   const int g = threadIdx.x % G;
   const int t = min((int)threadIdx.x / G, TP);
   float2 *S = fct_sm + g;
@@ -602,8 +606,8 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
     }
     if (in) *reinterpret_cast<float2 *>(col + (size_t)row_of(i) * wp) = make_float2(v.y, v.x);
   };
-  // the spectral step on points k and H - k of both columns (and, in the first cycle, the
-  // sum of squares that sets the grid of the iterate)
+  // the spectral step on points k and H - k of both columns (and the sum of squares that sets
+  // the grid of the correction)
   float acc = 0.f;
   auto spectral = [&] {
     if (t < TP) {
@@ -619,7 +623,7 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
         }
         Quad q = dct_post(z, zn, tk);
         const float lk = __ldg(a.y.s2 + k), ln = __ldg(a.y.s2 + kn);
-        if (kc == 0 && k == 0 && ja == 0) a.ctrl->rho_mean[c] = -scale * q.ak;
+        if (k == 0 && ja == 0) a.ctrl->rho_mean[c] += -scale * q.ak;  // (one thread)
         q.ak = (k == 0 && ja == 0) ? 0.f : q.ak * __fdividef(scale, lk + lxa);
         q.bk = q.bk * __fdividef(scale, lk + lxb);
         q.an = k == 0 ? 0.f : q.an * __fdividef(scale, ln + lxa);
@@ -654,14 +658,16 @@ fct_cols_kernel(const __grid_constant__ FctArgs a, int kc) {
     if (t < TP)
       for (int i = t; i < H; i += TP) to_image(i, S[i * G]);
   }
-  if (kc == 0) {
+  if (kc == 0 || (kc == 1 && a.tight)) {
     acc = fct_block_sum(acc);
-    if (threadIdx.x == 0) atomicAdd(&a.ctrl->rnorm2[fct_grid_slot(c)], (double)acc);
+    if (threadIdx.x == 0) atomicAdd(&a.ctrl->rnorm2[fct_grid_slot(kc, c)], (double)acc);
   }
 }
 
-// Rows back: the correction e of G row pairs. The iterate is kept as two parts: the first
-// correction (rounded to the channel's grid) and the sum of the later ones, 1e-5 of it.
+// Rows back: the correction e of G row pairs. The iterate is the sum of its corrections, each
+// 1e-5 .. 1e-6 of the one before and kept as a part of its own: the first rounded to the channel's grid, and
+// for rtol < 1e-6 the second to one too, or its Laplacian is only known to 3e-7 of a smooth field of
+// 4096 x 4096 points. (A wider rtol does not need that, and the rounding could cost it a third cycle.)
 template <class F, bool BL>
 __global__ void __launch_bounds__(ceil_div(F::G_ROWS * F::TP, 32) * 32, blocks_per_sm(F::G_ROWS * F::TP))
 fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
@@ -675,7 +681,6 @@ fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
   const int g = threadIdx.x / TP, t = g < G ? (int)threadIdx.x - g * TP : TP;
   float2 *S = fct_sm + (g < G ? g : 0) * F::template Layout<1>::SLOTS;
   const int W = a.W, H = a.H;
-  const size_t plane = (size_t)H * W;
   const int ia = 2 * (blockIdx.x * G + g);
   const bool va = t < TP && ia < H, vb = t < TP && ia + 1 < H;
   const float *sa = a.spec + ((size_t)c * H + ia) * a.wp, *sb = sa + a.wp;
@@ -689,13 +694,15 @@ fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
     return z;
   };
   dft<F, BL, 1>(S, a.x, t, false, [&](auto &v, int j, auto step) { gather<decltype(step)::value>(v, j, packed); });
-  float *uh = a.uhi + c * plane, *ul = a.ulo + c * plane;
   constexpr float inv_len = 1.f / (float)F::LEN;
   float acc = 0.f;
   if (va) {
     const int half = (W + 1) / 2;
-    float *out = kc == 0 ? uh : ul;
-    const float grid = kc == 0 ? fct_grid(a.ctrl->rnorm2[fct_grid_slot(c)]) : 0.f;
+    // the third correction takes the place of its spectrum, row by row (which this block has read)
+    const int pitch = kc > 1 ? a.wp : W;
+    float *out = (kc == 0 ? a.uhi : kc == 1 ? a.ulo : a.spec) + (size_t)c * H * pitch;
+    const bool round = kc == 0 || (kc == 1 && a.tight);
+    const float grid = round ? fct_grid(a.ctrl->rnorm2[fct_grid_slot(kc, c)]) : 0.f;
     for (int m = t; m < half; m += TP) {
       const int j = 2 * m;
       const bool two = j + 1 < W;
@@ -708,16 +715,11 @@ fct_back_kernel(const __grid_constant__ FctArgs a, int kc) {
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         if (r == 1 && !vb) break;
-        const size_t row = (size_t)(ia + r) * W;
         float2 v = e[r];
-        if (kc == 0) v = make_float2(__fsub_rn(__fadd_rn(v.x, grid), grid), __fsub_rn(__fadd_rn(v.y, grid), grid));
+        if (round) v = make_float2(__fsub_rn(__fadd_rn(v.x, grid), grid), __fsub_rn(__fadd_rn(v.y, grid), grid));
         acc += v.x;
         if (two) acc += v.y;
-        if (kc > 1) {
-          const float2 l = ld_pair(ul + row, j, W);
-          v = make_float2(v.x + l.x, v.y + l.y);
-        }
-        st_pair(out + row, j, W, v);
+        st_pair(out + (size_t)(ia + r) * pitch, j, W, v);
       }
     }
   }
