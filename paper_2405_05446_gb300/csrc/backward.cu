@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kBwdThreads, Q <= 6 ? 6 : 4) raster_backward_k
   __shared__ int s_pos[kBwdThreads / 32][32];     // place in the tile's list
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned ntiles = a.ctrl->n_active;
-  if (blockIdx.x >= ntiles || a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // no sorted list
+  if (blockIdx.x >= ntiles || a.ctrl->gave_up) return;  // no sorted list
   const int tile = (int)a.active[blockIdx.x];
   const int tyi = tile / a.tiles_x, txi = tile - tyi * a.tiles_x;
   const int x0 = txi * kTile, y0 = tyi * kTile;

@@ -35,7 +35,7 @@ struct Ctrl {
   int n_visible;       // Gaussians that survived projection
   unsigned long long n_pairs;  // (tile, splat) pairs requested (uncapped)
   unsigned n_active;   // tiles with at least one pair
-  unsigned pad0;
+  int gave_up;         // a sort's wait ran out: no order, no pairs (whatever status already holds)
   int max_cycles;
   int channels;
   int iter;            // cycle index when the cycle loop runs as a graph
@@ -110,6 +110,13 @@ struct LaunchScope {
 
 __device__ __forceinline__ void set_status(Ctrl *c, int code) {
   atomicCAS(&c->status, GDGS_OK, code);
+}
+// A bounded wait ran out. The status may hold an earlier error (a capacity overflow, a non-finite
+// parameter), so the kernels that follow go by a flag of its own: without a sorted list they
+// would index with what an earlier call left in the workspace.
+__device__ __forceinline__ void give_up(Ctrl *c) {
+  set_status(c, GDGS_ERR_TIMEOUT);
+  c->gave_up = 1;
 }
 
 // Geometry of one multigrid level. Level l has ceil(N0 / 2^l) cells per side;

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kRasterThreads) raster_kernel(RasterArgs a) {
   __shared__ float4 s_splat[kRasterThreads / 32][4 + QP][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned ntiles = a.use_active ? a.ctrl->n_active : (unsigned)a.T;
-  if (blockIdx.x >= ntiles || a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // no sorted list
+  if (blockIdx.x >= ntiles || a.ctrl->gave_up) return;  // no sorted list
   const int tile = a.use_active ? (int)a.active[blockIdx.x] : (int)blockIdx.x;
   const int tyi = tile / a.tiles_x, txi = tile - tyi * a.tiles_x;
   const int x0 = txi * kTile, y0 = tyi * kTile;

@@ -131,7 +131,6 @@ __global__ void __launch_bounds__(kHistThreads) depth_hist_kernel(DepthSort a, S
 template <int THREADS, int ITEMS, int BITS, int kKind>
 __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pass_kernel(SortPass a) {
   griddep_enter();
-  if (a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // an earlier pass gave up
   constexpr int kWarps = THREADS / 32, kKeys = THREADS * ITEMS;
   constexpr unsigned kMask = (1u << BITS) - 1u;
   static_assert(THREADS >= 256 && THREADS % 32 == 0, "a thread per digit");
@@ -145,7 +144,8 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
   uint2 *const row = wcnt + w * 256;
   uint16_t *const head = reinterpret_cast<uint16_t *>(wcnt);
   const unsigned lt = lanemask_lt();
-  if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
+  // (one thread looks: a block leaves as a whole, also when another one gives up meanwhile)
+  if (tid == 0) s_tile = a.ctrl->gave_up ? ~0u : atomicAdd(a.ticket, 1u);
   for (;;) {
     for (int t = tid; t < kWarps * 256; t += THREADS) wcnt[t] = make_uint2(0u, 0u);
     __syncthreads();
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
           sum += s[k] - 1u;
         }
         if (!done && ++polls > kLookBackLimit) {  // give up; the guard below keeps writes in bounds
-          set_status(a.ctrl, GDGS_ERR_TIMEOUT);
+          give_up(a.ctrl);
           done = true;
         }
         if (done) base += sum;
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
           go = go && !done;
         }
         if (!done && ++polls > kLookBackLimit) {
-          set_status(a.ctrl, GDGS_ERR_TIMEOUT);
+          give_up(a.ctrl);
           done = true;
         }
         if (!go && !done) __nanosleep(64);
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kBinBlock) count_kernel(BinArgs a) {
   griddep_enter();
   const int64_t i = (int64_t)blockIdx.x * kBinBlock + threadIdx.x;
   unsigned long long s = 0;
-  if (i < a.n && a.ctrl->status != GDGS_ERR_TIMEOUT) {  // (then there is no order)
+  if (i < a.n && !a.ctrl->gave_up) {  // (then there is no order)
     const uint32_t g = a.order[i];
     const uint2 rc = a.rect[g];
     if (rect_tiles(rc)) s = tiles_hit(a, g, rc);
@@ -492,7 +492,7 @@ __device__ __forceinline__ int owner(unsigned incl, unsigned i) {
 // clears what its first pass publishes.
 __global__ void __launch_bounds__(kBinBlock) emit_kernel(BinArgs a, int nb) {
   griddep_enter();
-  if (a.ctrl->status == GDGS_ERR_TIMEOUT) return;  // no order
+  if (a.ctrl->gave_up) return;  // no order
   __shared__ Footprint s_f[kBinBlock];
   __shared__ unsigned s_bins[4][256];
   const int tid = threadIdx.x, lane = tid & 31, w0 = tid & ~31;
