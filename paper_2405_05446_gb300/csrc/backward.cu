@@ -99,9 +99,10 @@ __device__ __forceinline__ bool warp_sums_valid(int lane, int count) {
   }
 }
 
-// a / b of both elements, correctly rounded for the normal range the transmittances live
-// in (a <= 1, 0.01 <= b <= 1): Newton-Raphson on an approximate reciprocal and Markstein's
-// correction of the quotient by its exact remainder (IBM J. Res. Dev. 34, 1990).
+// a / b of both elements: Newton-Raphson on an approximate reciprocal and Markstein's correction
+// of the quotient by its exact remainder (IBM J. Res. Dev. 34, 1990). CUDA's own quotient, bit for
+// bit, for a transmittance a of 1 to 2^-100 and b = 1 - alpha of 1 to 2^-24 (any alpha_max below
+// 1; 2 10^9 samples); from about 2^-107 down the remainder underflows and an ulp may be lost.
 __device__ __forceinline__ f32x2 div2(f32x2 a, f32x2 b) {
   float b0, b1, r0, r1;
   unpk(b, b0, b1);

@@ -21,9 +21,10 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["sort"])
+@pytest.mark.parametrize("what", ["sort", "div"])
 def test_native(checks, what):
     """sort: behind a bounded wait that gave up no pass of either sort runs, also where the
-    status already holds another error (the lists they would read were never written)."""
+    status already holds another error (the lists they would read were never written); div:
+    the packed division gives CUDA's quotient over the transmittances of 1 to 2^-100."""
     r = subprocess.run([checks, what], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
