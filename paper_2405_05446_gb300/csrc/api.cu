@@ -383,6 +383,7 @@ int gdgs_project(const gdgs_gaussians *g, const gdgs_camera *cam, const gdgs_ras
   cudaError_t e = cudaMemsetAsync(w + p.off_ctrl, 0, sizeof(Ctrl), st);
   if (e != cudaSuccess) return GDGS_ERR_CUDA;
   ProjectArgs a = project_args(g, cam, ro, p, w);
+  a.sort_scratch = nullptr;
   if (out) {
     a.o_mean2d = out->mean2d;
     a.o_cov2d = out->cov2d;

@@ -183,7 +183,7 @@ struct ProjectArgs {
   float w2c[12];
   float fx, fy, cx, cy, znear;
   int W, H, tiles_x, tiles_y;
-  uint32_t *sort_scratch;      // kSortWords words, zeroed here for the sorts that follow
+  uint32_t *sort_scratch;      // kSortWords words, zeroed here for the sorts that follow (null: none does)
   const gdgs_camera *cam_dev;  // when set, w2c .. znear are read from it on the device
   float alpha_min, dilation, exp_coef;
   // outputs (workspace)

@@ -83,10 +83,13 @@ __device__ __forceinline__ uint32_t depth_lo_digit(FF t) {
   return (uint32_t)fminf(fmaxf(q, 0.f), 255.f);
 }
 
+// kSorts: the sorts' counts are cleared for them (alone, project_1m takes 1 % less without).
+template <bool kSorts>
 __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   griddep_enter();
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < kSortWords; t += gridDim.x * blockDim.x)
-    a.sort_scratch[t] = 0u;
+  if (kSorts)
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < kSortWords; t += gridDim.x * blockDim.x)
+      a.sort_scratch[t] = 0u;
   if (a.cam_dev) {  // camera from device memory (a graph replays for any camera)
     const gdgs_camera *cd = a.cam_dev;
 #pragma unroll
@@ -230,7 +233,7 @@ cudaError_t launch_project(const ProjectArgs &a, cudaStream_t st) {
   if (a.n == 0) return cudaSuccess;
   const int threads = 256;
   const unsigned blocks = (unsigned)((a.n + threads - 1) / threads);
-  { LaunchScope ls_("project", st); launch_k(project_kernel, blocks, threads, 0, st, a); }
+  { LaunchScope ls_("project", st); launch_k(a.sort_scratch ? project_kernel<true> : project_kernel<false>, blocks, threads, 0, st, a); }
   return cudaGetLastError();
 }
 
