@@ -198,7 +198,8 @@ GDGS_API const char *gdgs_status_string(int status);
 
 /* Bytes of device workspace needed by any call below for n Gaussians, `channels`
  * channels and a width x height image (n = 0 sizes a Poisson-only workspace).
- * NULL options mean the defaults. Returns 0 if an argument is out of range. */
+ * NULL options mean the defaults. Returns 0 if an argument is out of range. The size
+ * belongs to the build of the library: ask for it, do not store it. */
 GDGS_API size_t gdgs_workspace_size(int64_t n, int32_t channels, int32_t width, int32_t height,
                            const gdgs_raster_opts *ropts, const gdgs_solver_opts *sopts);
 

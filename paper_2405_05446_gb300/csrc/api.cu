@@ -94,28 +94,40 @@ bool make_plan(int64_t n, int C, int W, int H, const gdgs_raster_opts &ro,
   // the cached coarse factor sits at a fixed offset with room for the largest
   // coarsest grid, so workspaces laid out for other sizes never overwrite it
   p->off_coarse = cv.take(kCoarseTagBytes + sizeof(double) * (size_t)kMaxCoarse * kMaxCoarse);
-  p->off_sub = cv.take(sizeof(Ctrl) * (size_t)C);
+  if (n == 0) p->off_sub = cv.take(sizeof(Ctrl) * (size_t)C);
+  p->off_range = cv.take(8 * (size_t)p->T);
+  p->off_active = cv.take(4 * (size_t)p->T);
+  p->off_mask = cv.take((size_t)p->T);
+  size_t sorts_end = 0;
   if (n > 0) {
     p->off_smean = cv.take(16 * (size_t)n);
     p->off_sconic = cv.take(16 * (size_t)n);
     p->off_rect = cv.take(8 * (size_t)n);
     for (int b = 0; b < 2; ++b) {
-      p->off_dkey[b] = cv.take(4 * (size_t)n);
-      p->off_dval[b] = cv.take(4 * (size_t)n);
       p->off_pkey[b] = cv.take(4 * (size_t)p->pair_cap);
       p->off_pval[b] = cv.take(4 * (size_t)p->pair_cap);
     }
-    p->off_dlo = cv.take(4 * (size_t)n);
-    p->off_hist = cv.take(4 * std::max(sort_state_words(n, kDepthTile), sort_state_words(cap, kPairTile)));
-    p->off_sort = cv.take(4 * kSortWords);
     p->off_blocksum = cv.take(8 * (size_t)((n + kBinBlock - 1) / kBinBlock + 2));
+    // The backward's 48 bytes per Gaussian begin on the six arrays of the depth sort, which end
+    // with the forward. What the sorts publish and count is live from the projection to the last
+    // pass only and begins on the rest of the backward's, the channels' control blocks, the maps and
+    // the solver's arrays: only the workspace of an image below a tile is larger for it.
+    p->off_dsplat = cv.cur;
+    for (int b = 0; b < 2; ++b) {
+      p->off_dkey[b] = cv.take(4 * (size_t)n);
+      p->off_dval[b] = cv.take(4 * (size_t)n);
+    }
+    p->off_dlo = cv.take(4 * (size_t)n);
     p->off_gtiles = cv.take(4 * (size_t)n);
+    Carver sorts = cv;
+    p->off_sort = sorts.take(4 * sort_words(p->T));
+    p->off_hist = sorts.take(4 * std::max(sort_state_words(n, kDepthTile, kDepthDigits, kSortPasses),
+                                          sort_state_words(cap, kPairTile, pair_digits(pair_digit(p->T)), pair_passes(p->T))));
+    sorts_end = sorts.cur;
+    cv.take(24 * (size_t)n);
+    p->off_sub = cv.take(sizeof(Ctrl) * (size_t)C);
     p->off_maps = cv.take(4 * (size_t)C * 2 * W * H);
-    p->off_dsplat = cv.take(48 * (size_t)n);
   }
-  p->off_range = cv.take(8 * (size_t)p->T);
-  p->off_active = cv.take(4 * (size_t)p->T);
-  p->off_mask = cv.take((size_t)p->T);
   const size_t plane0 = (size_t)W * H * C * sizeof(float);
   p->off_rho = cv.take(plane0);
   p->off_uhi = cv.take(plane0);
@@ -129,7 +141,7 @@ bool make_plan(int64_t n, int C, int W, int H, const gdgs_raster_opts &ro,
     p->off_lf[l] = cv.take(b);
     p->off_luo[l] = cv.take(b);
   }
-  p->total = cv.cur;
+  p->total = std::max(cv.cur, sorts_end);
   return true;
 }
 
@@ -215,6 +227,7 @@ ProjectArgs project_args(const gdgs_gaussians *g, const gdgs_camera *cam,
   a.key = (uint32_t *)(ws + p.off_dkey[0]);  // sorted in place by the depth sort
   a.key_lo = (uint32_t *)(ws + p.off_dlo);
   a.sort_scratch = (uint32_t *)(ws + p.off_sort);
+  a.sort_words = sort_words(p.T);
   a.rect = (uint2 *)(ws + p.off_rect);
   a.ctrl = (Ctrl *)(ws + p.off_ctrl);
   return a;
@@ -247,7 +260,7 @@ cudaError_t raster_path(const gdgs_gaussians *g, const gdgs_camera *cam,
     ds.key_lo = (const uint32_t *)(ws + p.off_dlo);
     ds.n = (unsigned)g->n;
     ds.state = state;
-    ds.scratch = {scratch, scratch + 2 * kSortPasses * 256};
+    ds.scratch = depth_scratch(scratch);
     ds.range = range;
     ds.tile_mask = mk;
     ds.T = p.T;
@@ -269,7 +282,7 @@ cudaError_t raster_path(const gdgs_gaussians *g, const gdgs_camera *cam,
     b.tiles = (uint32_t *)(ws + p.off_gtiles);
     b.pkey = (uint32_t *)(ws + p.off_pkey[0]);
     b.pval = pv[0];
-    b.bins = scratch + kSortPasses * 256;
+    b.bins = pair_scratch(scratch).bins;
     b.sort_state = state;
     b.ctrl = ctrl;
     e = launch_emit_pairs(b, st);
@@ -284,7 +297,7 @@ cudaError_t raster_path(const gdgs_gaussians *g, const gdgs_camera *cam,
     ps.cap = p.pair_cap;
     ps.T = p.T;
     ps.state = state;
-    ps.scratch = {scratch + kSortPasses * 256, scratch + 2 * kSortPasses * 256 + 8};
+    ps.scratch = pair_scratch(scratch);
     ps.range = range;
     ps.active = active;
     ps.tile_mask = mk;

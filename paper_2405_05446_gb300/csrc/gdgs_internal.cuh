@@ -21,7 +21,7 @@ constexpr int kDepthThreads = 256, kDepthItems = 8, kDepthTile = kDepthThreads *
 constexpr int kPairThreads = 256, kPairItems = 10, kPairTile = kPairThreads * kPairItems;
 constexpr int kHistThreads = 512, kHistGrid = 304, kSortGrid = 1216, kEmitGrid = 912;
 constexpr int kSortPasses = 5;  // of the depth sort; the pair sort has at most 4
-constexpr int kSortWords = 2 * (kSortPasses * 256 + 8);  // both sorts' digit counts and tickets
+constexpr int kDepthDigits = 256;
 constexpr int kBinBlock = 256;  // Gaussians per block of the pair count and emission
 constexpr uint32_t kInvalidKey = 0xFFFFFFFFu;
 
@@ -142,13 +142,13 @@ struct Plan {
   size_t off_smean, off_sconic, off_rect;              // projected splats [n]
   size_t off_dkey[2], off_dval[2];                     // depth sort [n]
   size_t off_dlo;                                      // depth sort secondary key [n]
-  size_t off_hist, off_sort;                           // sorts: status words; counts and tickets
+  size_t off_hist, off_sort;                           // sorts: published words; counts and tickets (shared, make_plan)
   size_t off_blocksum;                                 // scan partials
   size_t off_gtiles;                                   // tiles per depth-ordered Gaussian
   size_t off_pkey[2], off_pval[2];                     // pairs [pair_cap]
   size_t off_range, off_active, off_mask;              // per tile
   size_t off_maps;                                     // [C][2][H][W]
-  size_t off_dsplat;                                   // backward: [n][6]
+  size_t off_dsplat;                                   // backward: [n][6] (shared, make_plan)
   size_t off_rho, off_uhi, off_ulo, off_e0, off_r[2];  // level 0 [C][H][W]
   size_t off_lu[kMaxLevels], off_lf[kMaxLevels];       // levels >= 1: down-pass u, f
   size_t off_luo[kMaxLevels];                          // levels >= 1: up-pass u (never in place)
@@ -183,7 +183,8 @@ struct ProjectArgs {
   float w2c[12];
   float fx, fy, cx, cy, znear;
   int W, H, tiles_x, tiles_y;
-  uint32_t *sort_scratch;      // kSortWords words, zeroed here for the sorts that follow (null: none does)
+  uint32_t *sort_scratch;      // [sort_words], zeroed here for the sorts that follow (null: none does)
+  unsigned sort_words;
   const gdgs_camera *cam_dev;  // when set, w2c .. znear are read from it on the device
   float alpha_min, dilation, exp_coef;
   // outputs (workspace)
@@ -201,13 +202,14 @@ cudaError_t launch_project(const ProjectArgs &a, cudaStream_t st);
 
 // Radix sorts of 32-bit keys with 32-bit values, stable (sort.cu). The scratch is zeroed by
 // the projection; `state` holds what the tiles of two successive passes publish.
-size_t sort_state_words(long long keys, int tile);
+// (keys in tiles, digits of a pass; a sort of one pass has one set.)
+size_t sort_state_words(long long keys, int tile, int digits, int passes);
 struct SortState {
-  uint32_t *tile, *sum, *prefix;  // [tiles][256], [groups][256] twice
+  uint32_t *tile, *sum, *prefix;  // [tiles][digits], [groups][digits] twice
 };
 struct SortScratch {
-  uint32_t *bins;    // [kSortPasses][256]
-  unsigned *ticket;  // [kSortPasses]
+  uint32_t *bins;    // [passes][256]
+  unsigned *ticket;  // [passes]
 };
 
 enum { kSortPlain, kSortLow, kSortRanges };
@@ -266,6 +268,14 @@ inline int tile_bits(int T) {
 }
 inline int pair_passes(int T) { return (tile_bits(T) + 7) / 8; }
 inline int pair_digit(int T) { return (tile_bits(T) + pair_passes(T) - 1) / pair_passes(T); }
+__host__ __device__ inline int pair_digits(int digit) { return 1 << (digit < 5 ? 5 : digit); }  // (the passes have 5 bits or more)
+// Both sorts' digit counts and tickets: depth counts [kSortPasses][256], tickets [8] and [8], pair
+// counts [pair_passes][256] (the last pass's digits only).
+inline unsigned sort_words(int T) {
+  return kSortPasses * 256 + 16 + (pair_passes(T) - 1) * 256 + pair_digits(pair_digit(T));
+}
+inline SortScratch depth_scratch(uint32_t *w) { return {w, w + kSortPasses * 256}; }
+inline SortScratch pair_scratch(uint32_t *w) { return {w + kSortPasses * 256 + 16, w + kSortPasses * 256 + 8}; }
 
 // A tile's pairs: the sort leaves (~start, end), zero where there are none.
 __device__ __forceinline__ uint2 tile_range(const uint2 *range, int tile) {

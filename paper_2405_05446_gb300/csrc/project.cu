@@ -88,7 +88,7 @@ template <bool kSorts>
 __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   griddep_enter();
   if (kSorts)
-    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < kSortWords; t += gridDim.x * blockDim.x)
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < a.sort_words; t += gridDim.x * blockDim.x)
       a.sort_scratch[t] = 0u;
   if (a.cam_dev) {  // camera from device memory (a graph replays for any camera)
     const gdgs_camera *cd = a.cam_dev;

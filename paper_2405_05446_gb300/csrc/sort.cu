@@ -84,10 +84,10 @@ __device__ __forceinline__ unsigned scan_digits(unsigned v) {
 }
 
 // Clears what the tiles of a pass publish, by threads tid of nt.
-__device__ __forceinline__ void clear_state(const SortState &s, unsigned tiles, unsigned tid, unsigned nt) {
+__device__ __forceinline__ void clear_state(const SortState &s, unsigned tiles, unsigned digits, unsigned tid, unsigned nt) {
   const unsigned groups = (tiles + kGroup - 1) / kGroup;
-  for (unsigned t = tid; t < tiles * 256u; t += nt) s.tile[t] = 0u;
-  for (unsigned t = tid; t < groups * 256u; t += nt) s.sum[t] = s.prefix[t] = 0u;
+  for (unsigned t = tid; t < tiles * digits; t += nt) s.tile[t] = 0u;
+  for (unsigned t = tid; t < groups * digits; t += nt) s.sum[t] = s.prefix[t] = 0u;
 }
 
 // Digit counts of all passes of the depth sort (bins zeroed before), the cleared state of its
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kHistThreads) depth_hist_kernel(DepthSort a, S
   __shared__ unsigned sh[kSortPasses][256];
   const unsigned tid = blockIdx.x * kHistThreads + threadIdx.x, nt = gridDim.x * kHistThreads;
   for (int t = threadIdx.x; t < kSortPasses * 256; t += kHistThreads) (&sh[0][0])[t] = 0u;
-  clear_state(state, (a.n + kDepthTile - 1) / kDepthTile, tid, nt);
+  clear_state(state, (a.n + kDepthTile - 1) / kDepthTile, kDepthDigits, tid, nt);
   for (unsigned t = tid; t < (unsigned)a.T; t += nt) {
     a.range[t] = make_uint2(0u, 0u);
     a.tile_mask[t] = 0;
@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
   griddep_enter();
   constexpr int kWarps = THREADS / 32, kKeys = THREADS * ITEMS;
   constexpr unsigned kMask = (1u << BITS) - 1u;
+  constexpr int kDigits = 1 << BITS;
   static_assert(THREADS >= 256 && THREADS % 32 == 0, "a thread per digit");
   static_assert(ITEMS <= 32, "the list of run heads takes the counters' place, 16 bits a key");
   extern __shared__ uint32_t sort_sm[];
@@ -153,9 +154,9 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
     if (tile >= tiles) break;
     const unsigned first = tile * (unsigned)kKeys, cnt = min(n - first, (unsigned)kKeys);
     const unsigned group = tile / kGroup, member = tile % kGroup;
-    if (a.state_next.tile && tid < 256) {
-      a.state_next.tile[(size_t)tile * 256 + tid] = 0u;
-      if (member == 0) a.state_next.sum[group * 256 + tid] = a.state_next.prefix[group * 256 + tid] = 0u;
+    if (a.state_next.tile && tid < kDigits) {
+      a.state_next.tile[(size_t)tile * kDigits + tid] = 0u;
+      if (member == 0) a.state_next.sum[group * kDigits + tid] = a.state_next.prefix[group * kDigits + tid] = 0u;
     }
     // a warp's keys are consecutive: index = (warp, item, lane)
     const unsigned at = w * (32 * ITEMS) + lane;
@@ -192,14 +193,16 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
         wcnt[k * 256 + tid].x = c;
         c += x;
       }
-      st_status(&a.state.tile[(size_t)tile * 256 + tid], 1u + c);
-      atomicAdd(&a.state.sum[group * 256 + tid], (1u << kGroupBits) + c);
+      if (tid < kDigits) {
+        st_status(&a.state.tile[(size_t)tile * kDigits + tid], 1u + c);
+        atomicAdd(&a.state.sum[group * kDigits + tid], (1u << kGroupBits) + c);
+      }
     }
     const unsigned ex = scan_digits<THREADS>(c);
     unsigned base = 0;
     if (group == 0) {  // uniform: the first group starts at the digits' places
       __syncthreads();
-      base = scan_digits<THREADS>(tid < 256 ? a.bins[tid] : 0u);
+      base = scan_digits<THREADS>(tid < kDigits ? a.bins[tid] : 0u);
     }
     if (tid < 256) s_first[tid] = ex;
     __syncthreads();
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
         uint32_t s[kGroup - 1];
 #pragma unroll
         for (int k = 0; k < kGroup - 1; ++k)
-          s[k] = k < (int)member ? ld_status(&a.state.tile[(size_t)(tile - 1 - k) * 256 + tid]) : 1u;
+          s[k] = k < (int)member ? ld_status(&a.state.tile[(size_t)(tile - 1 - k) * kDigits + tid]) : 1u;
         unsigned sum = 0;
         done = true;
 #pragma unroll
@@ -238,9 +241,9 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
         uint32_t pre[kLookBack], sum[kLookBack];
 #pragma unroll
         for (int k = 0; k < kLookBack; ++k) {
-          pre[k] = g - k >= 0 ? ld_status(&a.state.prefix[(g - k) * 256 + tid]) : 0u;
+          pre[k] = g - k >= 0 ? ld_status(&a.state.prefix[(g - k) * kDigits + tid]) : 0u;
           // (group 0: its prefix, which has the smaller digits' keys)
-          sum[k] = g - k > 0 ? ld_status(&a.state.sum[(g - k) * 256 + tid]) : 0u;
+          sum[k] = g - k > 0 ? ld_status(&a.state.sum[(g - k) * kDigits + tid]) : 0u;
         }
         bool go = true;
 #pragma unroll
@@ -262,7 +265,7 @@ __global__ void __launch_bounds__(THREADS, kSortThreadsPerSm / THREADS) sort_pas
         }
         if (!go && !done) __nanosleep(64);
       }
-      if (member == kGroup - 1) st_status(&a.state.prefix[group * 256 + tid], kPrefix | ((base + c) & ~kPrefix));
+      if (member == kGroup - 1) st_status(&a.state.prefix[group * kDigits + tid], kPrefix | ((base + c) & ~kPrefix));
       s_out[tid] = base - ex;
     }
     if (kKind == kSortRanges && tid == 0) s_heads = 0;
@@ -498,7 +501,7 @@ __global__ void __launch_bounds__(kBinBlock) emit_kernel(BinArgs a, int nb) {
   const int tid = threadIdx.x, lane = tid & 31, w0 = tid & ~31;
   for (int t = tid; t < 4 * 256; t += kBinBlock) (&s_bins[0][0])[t] = 0u;
   const unsigned np = item_count(&a.ctrl->n_pairs, a.pair_cap);
-  clear_state(a.state, (np + kPairTile - 1) / kPairTile, blockIdx.x * kBinBlock + tid, gridDim.x * kBinBlock);
+  clear_state(a.state, (np + kPairTile - 1) / kPairTile, pair_digits(a.digit), blockIdx.x * kBinBlock + tid, gridDim.x * kBinBlock);
   const unsigned mask = (1u << a.digit) - 1u, full = 0xffffffffu;
   for (int block = blockIdx.x; block < nb; block += gridDim.x) {
     const int64_t i = (int64_t)block * kBinBlock + tid;
@@ -607,18 +610,19 @@ cudaError_t launch_pair_pass(const SortPass &a, int digit, unsigned tiles, cudaS
 
 unsigned pair_tiles(unsigned cap) { return (unsigned)(((unsigned long long)cap + kPairTile - 1) / kPairTile); }
 
-// The words of one of two successive passes over at most `tiles` tiles.
-SortState sort_state(uint32_t *base, int which, unsigned tiles) {
+// The words of one of two successive passes over at most `tiles` tiles (nobody reads those of
+// a single one: one set for all passes).
+SortState sort_state(uint32_t *base, int which, unsigned tiles, int digits) {
   const size_t groups = (tiles + kGroup - 1) / kGroup;
-  uint32_t *p = base + which * (size_t)256 * (tiles + 2 * groups);
-  return {p, p + (size_t)256 * tiles, p + (size_t)256 * (tiles + groups)};
+  uint32_t *p = base + (tiles > 1 ? which : 0) * digits * (tiles + 2 * groups);
+  return {p, p + digits * tiles, p + digits * (tiles + groups)};
 }
 
 }  // namespace
 
-size_t sort_state_words(long long keys, int tile) {
+size_t sort_state_words(long long keys, int tile, int digits, int passes) {
   const size_t tiles = (size_t)((keys + tile - 1) / tile), groups = (tiles + kGroup - 1) / kGroup;
-  return 2 * 256 * (tiles + 2 * groups);
+  return (tiles > 1 ? std::min(passes, 2) : 1) * digits * (tiles + 2 * groups);
 }
 
 cudaError_t sort_depth(const DepthSort &s, cudaStream_t st) {
@@ -627,7 +631,7 @@ cudaError_t sort_depth(const DepthSort &s, cudaStream_t st) {
   {
     LaunchScope ls_("radix_hist", st);
     launch_k(depth_hist_kernel, std::min<unsigned>((s.n + 4 * kHistThreads - 1) / (4 * kHistThreads), kHistGrid),
-             kHistThreads, 0, st, s, sort_state(s.state, 0, tiles));
+             kHistThreads, 0, st, s, sort_state(s.state, 0, tiles, kDepthDigits));
   }
   for (int p = 0; p < kSortPasses; ++p) {
     SortPass a{};
@@ -640,8 +644,8 @@ cudaError_t sort_depth(const DepthSort &s, cudaStream_t st) {
     a.shift = p ? 8 * (p - 1) : 0;
     a.bins = s.scratch.bins + 256 * p;
     a.ticket = s.scratch.ticket + p;
-    a.state = sort_state(s.state, p & 1, tiles);
-    if (p + 1 < kSortPasses) a.state_next = sort_state(s.state, ~p & 1, tiles);
+    a.state = sort_state(s.state, p & 1, tiles, kDepthDigits);
+    if (p + 1 < kSortPasses) a.state_next = sort_state(s.state, ~p & 1, tiles, kDepthDigits);
     a.ctrl = s.ctrl;
     const cudaError_t e = p ? launch_pass<kDepthThreads, kDepthItems, 8, kSortPlain>(a, tiles, st)
                             : launch_pass<kDepthThreads, kDepthItems, 8, kSortLow>(a, tiles, st);
@@ -665,8 +669,8 @@ cudaError_t sort_pairs(const PairSort &s, cudaStream_t st) {
     a.shift = p * digit;
     a.bins = s.scratch.bins + 256 * p;
     a.ticket = s.scratch.ticket + p;
-    a.state = sort_state(s.state, p & 1, tiles);
-    if (p + 1 < passes) a.state_next = sort_state(s.state, ~p & 1, tiles);
+    a.state = sort_state(s.state, p & 1, tiles, pair_digits(digit));
+    if (p + 1 < passes) a.state_next = sort_state(s.state, ~p & 1, tiles, pair_digits(digit));
     a.ctrl = s.ctrl;
     a.range = s.range;
     a.active = s.active;
@@ -681,7 +685,7 @@ cudaError_t sort_pairs(const PairSort &s, cudaStream_t st) {
 cudaError_t launch_emit_pairs(const BinArgs &b, cudaStream_t st) {
   if (b.n == 0) return cudaSuccess;
   BinArgs a = b;
-  a.state = sort_state(b.sort_state, 0, pair_tiles(b.pair_cap));
+  a.state = sort_state(b.sort_state, 0, pair_tiles(b.pair_cap), pair_digits(pair_digit(b.T)));
   a.passes = pair_passes(b.T);
   a.digit = pair_digit(b.T);
   const int nb = (int)((a.n + kBinBlock - 1) / kBinBlock);

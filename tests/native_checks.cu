@@ -51,7 +51,9 @@ static int run_sort(bool gave_up) {
   Buf<float4> d_mean(n), d_conic(n);
   Buf<uint2> d_rect(n), range(T, 0xff);
   Buf<uint32_t> k0(n), k1(n), v0(n), v1(n), d_lo(n), pk0(cap), pk1(cap), pv0(cap), pv1(cap), tiles(n), active(T);
-  Buf<uint32_t> state(std::max(sort_state_words(n, kDepthTile), sort_state_words(cap, kPairTile))), scratch(kSortWords);
+  Buf<uint32_t> state(std::max(sort_state_words(n, kDepthTile, kDepthDigits, kSortPasses),
+                               sort_state_words(cap, kPairTile, pair_digits(pair_digit(T)), pair_passes(T))));
+  Buf<uint32_t> scratch(sort_words(T));
   Buf<uint8_t> mask(T, 0xff);
   Buf<unsigned long long> blocksum((n + kBinBlock - 1) / kBinBlock + 2);
   Buf<Ctrl> ctrl(1);
@@ -70,18 +72,18 @@ static int run_sort(bool gave_up) {
   ds.key_lo = d_lo.p;
   ds.n = n;
   ds.state = state.p;
-  ds.scratch = {scratch.p, scratch.p + 2 * kSortPasses * 256};
+  ds.scratch = depth_scratch(scratch.p);
   ds.range = range.p, ds.tile_mask = mask.p, ds.T = T, ds.ctrl = ctrl.p;
   BinArgs b{};
   b.order = v1.p, b.rect = d_rect.p, b.smean = d_mean.p, b.sconic = d_conic.p;
   b.alpha_min = 1.f / 255.f, b.n = n, b.tiles_x = tx, b.T = T, b.pair_cap = cap;
   b.blocksum = blocksum.p, b.tiles = tiles.p, b.pkey = pk0.p, b.pval = pv0.p;
-  b.bins = scratch.p + kSortPasses * 256, b.sort_state = state.p, b.ctrl = ctrl.p;
+  b.bins = pair_scratch(scratch.p).bins, b.sort_state = state.p, b.ctrl = ctrl.p;
   PairSort ps{};
   ps.key[0] = pk0.p, ps.key[1] = pk1.p, ps.val[0] = pv0.p, ps.val[1] = pv1.p;
   ps.n_dev = (const unsigned long long *)((char *)ctrl.p + offsetof(Ctrl, n_pairs));
   ps.cap = cap, ps.T = T, ps.state = state.p;
-  ps.scratch = {scratch.p + kSortPasses * 256, scratch.p + 2 * kSortPasses * 256 + 8};
+  ps.scratch = pair_scratch(scratch.p);
   ps.range = range.p, ps.active = active.p, ps.tile_mask = mask.p, ps.ctrl = ctrl.p;
   if (sort_depth(ds, 0) != cudaSuccess || launch_emit_pairs(b, 0) != cudaSuccess || sort_pairs(ps, 0) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess) {
@@ -93,7 +95,7 @@ static int run_sort(bool gave_up) {
   const auto rg = range.get();
   if (gave_up) {
     bool same = c.n_pairs == 0 && c.n_active == 0 && c.status == GDGS_ERR_CAPACITY && order == ones_n && pk == ones_c && pv == ones_c;
-    for (int i = 0; i < 8; ++i) same = same && sc[2 * kSortPasses * 256 + i] == 0u && sc[2 * kSortPasses * 256 + 8 + i] == 0u;
+    for (int i = 0; i < 16; ++i) same = same && sc[kSortPasses * 256 + i] == 0u;  // the tickets
     for (const uint2 &r : rg) same = same && r.x == 0u && r.y == 0u;
     if (!same) printf("a pass ran behind a wait that gave up\n");
     return same ? 0 : 1;
