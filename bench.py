@@ -162,16 +162,24 @@ def min_traffic_bytes(kernel: str, C: int, H: int, W: int, cycles: int, n_gauss:
     return 0.0
 
 
+def pass_names(prof: dict) -> dict:
+    """The profile with the direct solve's row passes under names of their own: the library
+    records a cycle's residual and correction side as mg0_down and mg0_up with either solver."""
+    if "fct_columns" not in prof:
+        return prof
+    return {{"mg0_down": "fct_rows", "mg0_up": "fct_back"}.get(k, k): v for k, v in prof.items()}
+
+
 def direct_bytes(kernel: str, C: int, H: int, W: int, cycles: int, n_gauss: int,
                  n_pairs: int) -> float:
     """Bytes per view of the direct solve's passes (one read of their inputs, one write of
     their outputs; `cycles` refinement cycles). The other kernels as in min_traffic_bytes."""
     px = C * H * W
-    if kernel == "mg0_down":     # rows: rho (and from the second cycle on u) in, spectrum out
+    if kernel == "fct_rows":     # rows: rho (and from the second cycle on u) in, spectrum out
         return px * (cycles * (4 + 4) + (cycles - 1) * 4)
     if kernel == "fct_columns":  # spectrum in and out
         return cycles * px * 8
-    if kernel == "mg0_up":       # rows back: spectrum in, correction out
+    if kernel == "fct_back":     # rows back: spectrum in, correction out
         return cycles * px * 8
     return min_traffic_bytes(kernel, C, H, W, cycles, n_gauss, n_pairs)
 
@@ -621,7 +629,7 @@ def main():
         flush.zero_()
         G.render_view(g, cam, mean, out, r.ws, ropts, sopts_prof)
     torch.cuda.synchronize()
-    prof = G.profile_end()
+    prof = pass_names(G.profile_end())
 
     if rank != 0:
         dist.destroy_process_group() if world > 1 else None
@@ -680,7 +688,7 @@ def main():
             "config": {"workload": args.workload, "description": WORKLOADS[args.workload],
                        "solver": {"nu1": sopts.nu1, "nu2": sopts.nu2, "omega": round(sopts.omega, 4),
                                   "coarse_max_dim": sopts.coarse_max_dim, "rtol": rtol,
-                                  "storage": args.storage},
+                                  "storage": "none (direct solve)" if direct else args.storage},
                        "global_batch": world, "seq_len": None, "parallelism": f"replicas x{world}",
                        "l2": "flushed between timed views (256 MB write)"},
             "mpix_per_s": value * W * H / 1e6,

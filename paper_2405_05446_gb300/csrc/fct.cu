@@ -313,6 +313,8 @@ cudaError_t run_fct(const PoissonArgs &a, const FctPlan &f, const float *rho, fl
   const int V = a.W % 4 == 0 ? 4 : 1;
   const long long nq = (long long)a.H * (a.W / V);
   const dim3 fg((unsigned)std::max<long long>(1, std::min<long long>((nq + 255) / 256, 608)), a.C);
+  // The profile's names of a cycle's residual side and correction side on the finest grid are those of
+  // the multigrid: callers find them there with either solver, and fct_columns tells which one ran.
   for (int k = 0; k < f.cycles; ++k) {
     {
       LaunchScope ls_("mg0_down", st);
