@@ -7,7 +7,6 @@
 namespace gdgs {
 
 constexpr int kFctMaxCycles = 3;      // refinement cycles of a direct solve
-constexpr int kFctMaxThreads = 768;
 
 // The transform of one side of the image: length n of the cosine transform, done by
 // complex FFTs of `len` points: len == n when the library has an FFT of that length,

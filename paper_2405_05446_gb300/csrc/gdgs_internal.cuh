@@ -382,8 +382,8 @@ __device__ __forceinline__ void store_pairs(const StagedSplat &st, float4 *s, in
   s[3 * stride] = make_float4(st.geo2.w, st.geo2.w, st.geo2.y, st.geo2.y);
 }
 
-// log2 of alpha (before its clamp) at a lane's two pixels, L - p2 + c0, operation by
-// operation as L - staged_exponent() of each; X and Y are the offsets to h.
+// log2 of alpha (before its clamp) at a lane's two pixels, L - p2 + c0 with the expanded
+// exponent X (A X + (B' Y + a)) + Y (C Y + b); X and Y are the offsets to h.
 __device__ __forceinline__ void staged_log2_alpha(const float4 *s, int stride, f32x2 fpx, f32x2 fpy, f32x2 &X, f32x2 &Y,
                                                   float &t0, float &t1) {
   const ulonglong2 h = *reinterpret_cast<const ulonglong2 *>(s);
@@ -395,14 +395,6 @@ __device__ __forceinline__ void staged_log2_alpha(const float4 *s, int stride, f
   const f32x2 u = fma2(ab.x, X, fma2(ab.y, Y, lc.x));
   const f32x2 p = fma2(X, u, mul2(Y, fma2(lc.y, Y, bl.x)));
   unpk(fma2(p, pk(-1.f, -1.f), bl.y), t0, t1);
-}
-
-// p2 - c0 at the pixel centre (fpx, fpy) relative to the tile origin.
-__device__ __forceinline__ float staged_exponent(const float4 &ge, const float4 &ge2, float fpx,
-                                                 float fpy, float &X, float &Y) {
-  X = fpx - ge.x;
-  Y = fpy - ge.y;
-  return fmaf(X, fmaf(ge.z, X, fmaf(ge.w, Y, ge2.z)), Y * fmaf(ge2.x, Y, ge2.w));
 }
 
 // Which splats reach a block of a 16 x 16 tile (the rasterisers' warps hold 8 x 8 pixels):
