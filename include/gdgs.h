@@ -132,9 +132,13 @@ typedef struct gdgs_raster_opts {
 /* Solver options (Sec. 2.1; the paper fixes no parameters).
  * With the default omega and coarse_max_dim and both sides in 2..4096 the system
  * is solved directly by cosine transforms in FP32, refined twice (a third time
- * when rtol is not met); nu1, nu2 and storage then change nothing, and max_cycles
- * bounds the refinement cycles. Any other omega or coarse_max_dim, other sizes
- * and large images whose sides have large prime factors take multigrid cycles. Both stop at the same residual.
+ * when rtol is not met, which reaches 1e-9, and 3e-8 where the field is the
+ * lowest mode of a large image); nu1, nu2 and storage then change nothing, and
+ * max_cycles bounds the refinement cycles. Any other omega or coarse_max_dim,
+ * other sizes, images so small or thin that the solve's tables do not fit the
+ * workspace beside them, and large images of even width with sides that have no
+ * transform of their own length (csrc/fct.cu) take multigrid cycles. Both stop at
+ * the same residual.
  *   nu1, nu2        red-black Gauss-Seidel sweeps before / after the coarse
  *                   correction, each in 1..3                         (2, 1)
  *   max_cycles      upper bound on cycles, 1..64                     (30)
@@ -169,7 +173,7 @@ enum { GDGS_STORAGE_F32 = 0, GDGS_STORAGE_BF16 = 1, GDGS_STORAGE_F16 = 2 };
 /* Filled by gdgs_sync_status() from the workspace after the stream has drained. */
 typedef struct gdgs_solve_stats {
   int32_t status;          /* device status word (a GDGS_* code) */
-  int32_t cycles;          /* V-cycles run by the last solve */
+  int32_t cycles;          /* refinement cycles or V-cycles run by the last solve */
   double rel_residual;     /* ||rho - L u||_2 / ||rho||_2 of the returned solution */
   double rho_norm;         /* ||rho||_2 over all channels */
   double mean_set[GDGS_MAX_CHANNELS]; /* per-channel mean that was imposed */
@@ -225,7 +229,7 @@ GDGS_API int gdgs_render_gradients(const gdgs_gaussians *g, const gdgs_camera *c
                           uint8_t *tile_mask, void *ws, size_t ws_bytes, void *stream);
 
 /* Step 3 (Eq. p2d): rho = div(grad_maps) with zero flux through the image border,
- * then solve the Neumann problem L u = rho by multigrid V-cycles and return
+ * then solve the Neumann problem L u = rho (gdgs_solver_opts) and return
  *   image  device [channels][height][width], mean(image[c]) = mean[c].
  * grad_maps  device [channels][2][height][width]; tile_mask as written by
  *            gdgs_render_gradients (tiles with mask 0 are read as zero), or NULL.

@@ -1,7 +1,7 @@
 // Direct Neumann solve (Eq. p2d) by cosine transforms, refined to the caller's rtol.
 // Measured on a GB300 against the multigrid cycles it takes over from: 1920x1080x3 from
-// maps 739 -> 210 us, 1355x757x3 (Bluestein) 783 -> 293 us, 3840x2160x1 1473 -> 275 us,
-// 128x96x1 218 -> 59 us; relative error of the image 1.5e-6 -> 1e-7 (1080p).
+// maps 744 -> 207 us, 1355x757x3 (Bluestein) 780 -> 292 us, 3840x2160x1 1400 -> 270 us,
+// 128x96x1 221 -> 55 us; relative error of the image 1.5e-6 -> 1e-7 (1080p).
 //
 // On the pixel grid the 5-point Neumann Laplacian is diagonal in the DCT-II modes of
 // the two sides (Sec. 2.1 lists Fourier-type solvers beside multigrid): with
@@ -20,8 +20,10 @@
 // A transform of n points works on two real sequences at once, packed as the real and
 // imaginary part of one complex FFT of n points (Makhoul's even-odd order), held in
 // shared memory. The FFT is mixed-radix Stockham, one radix-R butterfly set per thread
-// in registers between two barriers, in place. Sides with a prime factor above 13 use
-// Bluestein's chirp convolution on a length >= 2 n - 1 instead.
+// in registers between two barriers, in place. Sides that are not in the list of
+// fct_pass.cuh (83 even products of two or three radices up to 16 without 7, 11 and 13; no odd
+// side, and not 448 = 64 * 7 or 2000 = 16 * 125) use Bluestein's chirp convolution on a
+// length >= 2 n - 1 instead: two FFTs of that length per transform.
 #include <stdlib.h>
 
 #include <algorithm>

@@ -83,7 +83,8 @@ __device__ __forceinline__ uint32_t depth_lo_digit(FF t) {
   return (uint32_t)fminf(fmaxf(q, 0.f), 255.f);
 }
 
-// kSorts: the sorts' counts are cleared for them (alone, project_1m takes 1 % less without).
+// kSorts: the sorts' counts are cleared for them (the projection of 1M Gaussians alone takes 42.0
+// us without, 42.8 with).
 template <bool kSorts>
 __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   griddep_enter();

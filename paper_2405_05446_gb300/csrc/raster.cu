@@ -12,9 +12,8 @@
 // (hi, lo) pair becomes a grid part that pixel centres subtract exactly and a
 // remainder folded into the expanded exponent, so alpha keeps FP32 relative
 // precision anywhere in the image. alpha = 2^(L - p2) with L = log2(opacity)
-// (ex2.approx; k log2 e is folded into the conic at projection); splats whose
-// exponent already puts them below alpha_min (with a 1e-3 margin in the
-// exponent) are skipped without the exponential.
+// (ex2.approx; k log2 e is folded into the conic at projection), taken for every splat
+// whose ellipse reaches the warp's block.
 //
 // One CTA of 128 threads per tile; a warp holds an 8 x 8 pixel block and a lane two
 // pixels of one column, 4 rows apart, whose arithmetic runs as packed FP32 pairs
