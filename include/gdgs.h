@@ -10,8 +10,8 @@
  *      touching only the 16x16 tiles that some splat reaches (the field is
  *      sparse, Sec. 2.2);
  *   3. take the divergence (the Laplacian field, Sec. 1.5) and solve the Neumann
- *      Poisson problem Delta c = rho (Eq. p2d) with a linear-complexity multigrid
- *      solver (Sec. 2.1, Sec. 2.2 "Poisson Equation"), fixing the constant the
+ *      Poisson problem Delta c = rho (Eq. p2d) directly by cosine transforms or by
+ *      multigrid cycles (Sec. 2.1, Sec. 2.2 "Poisson Equation"), fixing the constant the
  *      Neumann problem leaves free ("with possible constant difference", Sec. 2.1)
  *      with a supplied per-channel mean.
  *
@@ -62,7 +62,7 @@ enum {
   GDGS_ERR_INVALID_ARG = 1,  /* bad pointer, size, option or alignment (host) */
   GDGS_ERR_WORKSPACE = 2,    /* workspace null, misaligned or too small (host) */
   GDGS_ERR_CUDA = 3,         /* a CUDA launch or copy failed (host) */
-  GDGS_ERR_NO_CONVERGE = 4,  /* multigrid hit max_cycles above rtol (device) */
+  GDGS_ERR_NO_CONVERGE = 4,  /* the solver hit its last cycle above rtol (device) */
   GDGS_ERR_NONFINITE = 5,    /* NaN/Inf in an input Gaussian or map (device) */
   GDGS_ERR_TIMEOUT = 6,      /* a bounded device-side wait gave up (device) */
   GDGS_ERR_CAPACITY = 7      /* more (tile, splat) pairs than the pair buffer holds (device) */
